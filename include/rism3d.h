@@ -229,8 +229,9 @@ RISM_API rism_status rism_potential_batched(rism_ctx* const* ctxs, int32_t count
  * is 0; k_tol <= 0 sums the whole half spectrum.  *k_cut (host, nullable)
  * receives the cut-off (0 = none).  c_k, h_k: device or host memory, each
  * nullable (h_k needs kappa > 0, RISM_E_INVALID otherwise).  The structure
- * factor runs on the GPU with FP32 phase tables reduced exactly modulo one
- * cycle and FP32 products with float-float sums.  Synchronises the
+ * factor runs on the tensor cores: FP32 phase tables reduced exactly modulo
+ * one cycle, split into FP16 slices whose leading products add up without
+ * rounding, and float-float sums over blocks of atoms.  Synchronises the
  * context's stream.  RISM_E_STATE before set_solute/set_solvent. */
 RISM_API rism_status rism_asymptotics_k(rism_ctx* ctx, double k_tol, double* c_k, double* h_k, double* k_cut);
 

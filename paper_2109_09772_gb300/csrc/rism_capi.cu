@@ -780,8 +780,7 @@ rism_status rism_asymptotics_k(rism_ctx* c, double k_tol, double* c_k, double* h
         ks.qs[k] = k < c->S ? c->qs[k] : 0.0;
         if (k < c->S) ks.qmax = std::max(ks.qmax, std::fabs(c->qs[k]));
     }
-    ks.qabs = 0.0;
-    for (int64_t i = 0; i < c->n; ++i) ks.qabs += std::fabs(c->h_raw[6 * i + 3]);
+    kspace_charge_plan(c->h_raw, c->n, ks);
     ks.kcut = k_tol > 0.0 ? kspace_kcut(ks, k_tol) : 0.0;
     if (k_cut) *k_cut = ks.kcut;
     if (!c_k && !h_k) return RISM_OK;
@@ -810,7 +809,10 @@ rism_status rism_asymptotics_k(rism_ctx* c, double k_tol, double* c_k, double* h
         }
         dev[k] = c->d_kstage[k];
     }
-    const size_t tb = kspace_table_bytes(c->n, c->g.nx, c->g.ny, c->g.nz);
+    int sms = 0;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess)
+        return cuda_fail(c, e, "device attribute");
+    const size_t tb = kspace_table_bytes(c->n, c->g.nx, c->g.ny, c->g.nz, ks, sms);
     if (tb > c->ktab_bytes) {
         cudaFree(c->d_ktab);
         c->d_ktab = nullptr;
@@ -826,7 +828,7 @@ rism_status rism_asymptotics_k(rism_ctx* c, double k_tol, double* c_k, double* h
         }
         cudaEventRecord(c->ev[0], c->st);
     }
-    if ((e = launch_kspace(c->t, c->gd, ks, c->d_ktab, dev[0], dev[1], c->o.wait_limit, c->st)) != cudaSuccess)
+    if ((e = launch_kspace(c->t, c->gd, ks, sms, c->d_ktab, dev[0], dev[1], c->o.wait_limit, c->st)) != cudaSuccess)
         return cuda_fail(c, e, "k-space kernels");
     if (timed) cudaEventRecord(c->ev[1], c->st);
     for (int k = 0; k < 2 && host; ++k)

@@ -223,11 +223,9 @@ static __device__ __noinline__ double f2d_special(uint32_t b) {
 }
 __device__ __forceinline__ double f2d_alu(float f) {
     const uint32_t b = __float_as_uint(f);
-    const uint32_t e = (b >> 23) & 0xffu;
-    if (__builtin_expect(e - 1u >= 254u, 0)) return f2d_special(b);
-    const unsigned long long r = ((unsigned long long)(b >> 31) << 63) | ((unsigned long long)(e + 896u) << 52) |
-                                 ((unsigned long long)(b & 0x7fffffu) << 29);
-    return __longlong_as_double((long long)r);
+    // all-ones or zero exponent: 2b - 2^24 >= 2^32 - 2^25
+    if (__builtin_expect((b << 1) - 0x01000000u >= 0xfe000000u, 0)) return f2d_special(b);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
 // Error-free sum of two floats: a + b = s + e exactly.

@@ -129,6 +129,27 @@ def test_ellipsoid13600_sampled(R):
     r.close()
 
 
+@pytest.mark.parametrize("charges", ["equal", "one_large", "tiny"])
+def test_accumulation_blocks(R, charges):
+    """1,500 atoms whose charges all add up at k = 0 (|Q| equal: the exact accumulator holds 224 atoms, seven blocks),
+    one of which is 1,000 times the rest, or that are 1e-12 e: the blocks, the operand scale and the running sums."""
+    w = I.small_workload(n_atoms=1500, n=(30, 18, 21), h=0.9, seed=14, ions=True, lj_rcut=4.0, net=1.0)
+    q = w.solute.q
+    if charges == "equal":
+        q[:] = 0.75
+    elif charges == "one_large":
+        q[700] = 350.0
+    else:
+        q *= 1e-12
+    r = R.from_workload(w, method=R.METHOD_DIRECT, precision=R.PREC_FP32)
+    c, h, _ = r.asymptotics_k(0.0)
+    got = {"c": c.cpu().numpy().reshape(r.S, -1), "h": h.cpu().numpy().reshape(r.S, -1)}
+    r.close()
+    ref = O.kspace(O.Problem.from_workload(w))
+    for k in ("c", "h"):
+        _check(got[k], ref[k], f"{charges} {k}")
+
+
 def test_edge_cases(R):
     w = I.small_workload(n_atoms=10, n=(12, 10, 9), h=0.5, seed=2, ions=False)
     r = R.from_workload(w, method=R.METHOD_DIRECT, precision=R.PREC_FP32)
