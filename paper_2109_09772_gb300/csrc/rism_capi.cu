@@ -32,7 +32,10 @@ struct rism_ctx {
     int S = 0;
     double qs[kMaxSites] = {}, sigs[kMaxSites] = {}, epss[kMaxSites] = {}, rho[kMaxSites] = {};
     int is_ion[kMaxSites] = {};
-    bool have_solute = false, have_solvent = false, dirty = true;
+    bool have_solute = false, have_solvent = false;
+    // the per-pair tables and the tree (with its lists) are stale: built when a call first needs them (the
+    // reciprocal-space and all-space sums need only the tables)
+    bool dirty = true, tree_dirty = true;
     int64_t tree_calls = 0;  // treecode initializations of this context (the graph path starts at the second)
 
     // device state
@@ -180,11 +183,19 @@ rism_status ensure_tables(rism_ctx* c) {
             return cuda_fail(c, e, "setup kernel");
         c->setup_launches += 1;
     }
+    c->dirty = false;
+    return RISM_OK;
+}
+
+// The tables and, for the treecode, the tree of the current solute.
+rism_status ensure_tree(rism_ctx* c) {
+    rism_status s = ensure_tables(c);
+    if (s != RISM_OK || !c->tree_dirty) return s;
     if (c->o.method == RISM_METHOD_TREECODE) {
-        rism_status s = tree_prepare(c->tree, c->t, c->gd, c->ph, c->o, c->st, c->err);
+        s = tree_prepare(c->tree, c->t, c->gd, c->ph, c->o, c->st, c->err);
         if (s != RISM_OK) return s;
     }
-    c->dirty = false;
+    c->tree_dirty = false;
     return RISM_OK;
 }
 
@@ -291,7 +302,7 @@ rism_status rism_set_solute(rism_ctx* c, int64_t n, const double* xyz, const dou
     }
     c->n = n;
     c->have_solute = true;
-    c->dirty = true;
+    c->dirty = c->tree_dirty = true;
     ++c->solute_version;
     c->err.clear();
     return RISM_OK;
@@ -310,7 +321,7 @@ rism_status rism_set_solvent(rism_ctx* c, int32_t nsite, const double* q, const 
         c->is_ion[s] = (s < nsite && is_ion) ? (is_ion[s] != 0) : 0;
     }
     c->have_solvent = true;
-    c->dirty = true;
+    c->dirty = c->tree_dirty = true;
     c->err.clear();
     make_phys(c);  // beta, kappa, r_short are reported by rism_get_info from here on
     return RISM_OK;
@@ -417,7 +428,7 @@ rism_status rism_init(rism_ctx* c, double* u, double* c_lr, double* h_lr, double
     // one launch.
     const bool any_out = o.u || o.c || o.h;
     if (c->o.method == RISM_METHOD_TREECODE && any_out) ++c->tree_calls;
-    if (c->o.method == RISM_METHOD_TREECODE && c->dirty && c->n > 0 && any_out && c->tree_calls > 1) {
+    if (c->o.method == RISM_METHOD_TREECODE && c->tree_dirty && c->n > 0 && any_out && c->tree_calls > 1) {
         if ((s = reserve_tables(c)) != RISM_OK) return s;
         const bool tail = lj_tail && c->o.lj_mode != RISM_LJ_NONE;
         SoluteStep step{c->h_raw, c->d_raw, c->n, c->sigs, c->epss, c->o.lj_mode, c->o.lj_rcut, c->o.lj_tol,
@@ -437,7 +448,7 @@ rism_status rism_init(rism_ctx* c, double* u, double* c_lr, double* h_lr, double
             if (!retry) {
                 if (lj_tail)
                     for (int k = 0; k < c->S; ++k) lj_tail[k] = tail ? c->h_tail[k] : 0.0;
-                c->dirty = false;
+                c->dirty = c->tree_dirty = false;
                 c->setup_launches = 0;
                 if (c->o.debug_flags & 2) c->info.eval_ms = c->info.box_ms + c->info.far_ms + c->info.near_ms;
                 return RISM_OK;
@@ -445,7 +456,7 @@ rism_status rism_init(rism_ctx* c, double* u, double* c_lr, double* h_lr, double
             // a list outgrew its slots (now enlarged): rebuild through the regular path below
         }
     }
-    s = ensure_tables(c);
+    s = ensure_tree(c);
     if (s != RISM_OK) return s;
     c->info.launches = c->setup_launches;
     c->setup_launches = 0;
@@ -531,7 +542,7 @@ rism_status rism_potential_backward(rism_ctx* c, const double* g_u, const double
     void* outs[4] = {d_xyz, d_q, d_sigma, d_eps};
     for (void* p : outs)
         if (p && !is_device_ptr(p)) return fail(c, RISM_E_INVALID, "gradient outputs must be device memory");
-    rism_status s = ensure_tables(c);
+    rism_status s = ensure_tree(c);
     if (s != RISM_OK) return s;
     if (g_h && !(c->ph.kappa > 0.0)) g_h = nullptr;  // h is identically zero without ions
     s = adjoint_run(c->adj, c->tree, c->t, c->gd, c->ph, c->o, c->d_raw, c->sigs, c->epss, g_u, g_c, g_h, d_xyz,
@@ -608,7 +619,7 @@ rism_status rism_potential_batched(rism_ctx* const* ctxs, int32_t count, double*
         if (!again) {
             // the tables now match the uploaded solutes; the tree state is not reusable by rism_init
             // without a rebuild (its batch shape is the batch's), so mark every context dirty
-            for (int b = 0; b < count; ++b) ctxs[b]->dirty = true;
+            for (int b = 0; b < count; ++b) ctxs[b]->dirty = ctxs[b]->tree_dirty = true;
             return RISM_OK;
         }
     }

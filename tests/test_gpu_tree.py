@@ -386,3 +386,34 @@ def test_host_outputs_box_level_in_slabs_ordered(R):
             assert np.array_equal(out[k].cpu().numpy().reshape(S, M), host[i]), (step, k)
     for r in (rd, rh):
         r.close()
+
+
+@pytest.mark.parametrize("first", ["kspace", "lra"])
+def test_table_calls_leave_the_tree_to_the_next_evaluation(R, first):
+    """The reciprocal-space and all-space calls build only the per-pair tables: an evaluation, and a reverse pass,
+    of the same context afterwards see the new solute's tree (bit for bit those of a fresh context), also where an
+    earlier solute's tree was in place."""
+    import torch
+
+    a = I.small_workload(n_atoms=400, n=(48, 40, 36), h=0.5, seed=31, ions=True, lj_rcut=6.0, net=2.0)
+    b = I.small_workload(n_atoms=380, n=(48, 40, 36), h=0.5, seed=32, ions=True, lj_rcut=6.0, net=-1.0)
+    g = torch.randn((4, 36, 40, 48), dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    r = R.from_workload(a, method=R.METHOD_TREECODE, precision=R.PREC_FP32)
+    r.init()
+    for w in (b, a, b):
+        f = R.from_workload(w, method=R.METHOD_TREECODE, precision=R.PREC_FP32)
+        want, wgrad = f.init(), f.backward(g, g, g)
+        f.close()
+        for order in ("init", "backward"):
+            s = w.solute
+            r.set_solute(s.xyz, s.q, s.sigma, s.eps)
+            if first == "kspace":
+                r.asymptotics_k(0.0)
+            else:
+                r.lra_integral()
+            if order == "init":
+                got = r.init()
+                assert all(torch.equal(got[k], want[k]) for k in ("u", "c", "h"))
+            got = r.backward(g, g, g)
+            assert all(torch.equal(got[k], wgrad[k]) for k in wgrad)
+    r.close()
