@@ -424,7 +424,8 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     // enough CTAs to fill the GPU several times; at most one per row segment
     int chunks = (4 * 152 + ablocks - 1) / ablocks;
     chunks = max(1, min(chunks, min(nseg, 256)));
-    const int64_t need_part = (int64_t)chunks * n * 4;
+    const int tchunks = tree && o.method == RISM_METHOD_TREECODE ? tree_adjoint_chunks(n) : 0;
+    const int64_t need_part = (int64_t)max(chunks, tchunks) * n * 4;
     if (need_part > s->cap_part) {
         cudaFree(s->part);
         s->part = nullptr;
@@ -463,11 +464,11 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     const bool dh = g_h && ph.kappa > 0.0;
     bool tree_far = false;
     if (tree && o.method == RISM_METHOD_TREECODE) {
-        rism_status r = tree_adjoint_far(tree, t, g, ph, o, s->w, dh, s->part, st, err, tree_far);
+        rism_status r = tree_adjoint_far(tree, t, g, ph, o, s->w, dh, s->part, tchunks, st, err, tree_far);
         if (r != RISM_OK) return r;
     }
     if (tree_far) {
-        chunks = 1;  // one partial per atom, written in original atom order
+        chunks = tchunks;  // written in original atom order
     } else {
         dim3 grid(ablocks, chunks);
         if (dh) k_adj_far<true><<<grid, kAT, 0, st>>>(fa);

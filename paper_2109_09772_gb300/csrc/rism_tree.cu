@@ -5081,117 +5081,214 @@ __global__ void __launch_bounds__(32 * kListWarps) k_adj_lists(TBoxes tb, const 
     }
 }
 
-constexpr int kADThreads = 128;  // 4 threads per atom of a leaf
-constexpr int kADSub = kADThreads / kAL;
+constexpr int kADWarps = 8;     // warps per CTA: one group's targets in the lanes, the sources split over the warps
+constexpr int kADRows = 27;     // proxy rows per unit at most (whole planes)
 
-// One pair of the reverse far field: potential and radial factor of W1/d + Wk e^{-kappa d}/d.
-template <bool DH>
-__device__ __forceinline__ void adj_pair(float dx, float dy, float dz, float w1, float wk, float kap2, float kapg,
-                                         float& pq, float& px, float& py, float& pz) {
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    const float rr = rsqrt_approx(d2);
-    const float ri = d2 > 0.f ? rr : 0.f;  // a grid point on the atom: no term (d = 0 has no gradient)
-    float t1 = w1 * ri, tg = t1;
-    if (DH) {
-        const float d = d2 * ri;
-        const float tk = wk * ri * ex2_approx(kap2 * d);
-        t1 += tk;
-        tg = fmaf(tk, kapg * d, t1);
+// Units of work of a list entry: a plane of 16 x 16 grid points of a level-0 region, or a few planes of a box's
+// proxies (N1 x N1 each).  Both are rows along x at one (y, z).
+template <int N1>
+struct AdjUnit {
+    static constexpr int PU = kADRows / N1 > 0 ? kADRows / N1 : 1;      // proxy planes per unit
+    static constexpr int NU = (N1 + PU - 1) / PU;                         // units of a box
+    static constexpr int NP = (N1 + 1) / 2, NPG = kTB0 / 2;              // source pairs per proxy row, per grid row
+    static constexpr int REC = PU * N1 * NP > kTB0 * NPG ? PU * N1 * NP : kTB0 * NPG;  // pair records
+};
+
+// The sums of one target over the sources of a unit: potential, radial sums along x, y, z.
+struct AdjSums {
+    float q, x, y, z;
+};
+
+// One row of NP source pairs (two-wide: consecutive sources along x) against the warp's targets (one per lane), all at
+// offsets (dy, dz): every pair adds T = W1/d + Wk e^{-kappa d}/d to the potential and F = (W1 + Wk (1 + kappa d)
+// e^{-kappa d})/d^3 times its offset to the radial sums; along the row only x changes, so y and z take the row's sum of
+// F once.  Per pair 8 FMA-pipe operations and a reciprocal square root (DH: 14 and an exponential), a shared-memory
+// load of 16 bytes per two sources for all 32 targets.  ON: some target sits on a lattice point; a source at d = 0 has
+// no term.
+template <int NP, bool DH, bool ON>
+__device__ __forceinline__ void adj_row(const float4* rec, const f32x2 (&DX)[NP], float dy, float dz, f32x2 K2,
+                                        f32x2 KG, f32x2& PQ, f32x2& PX, AdjSums& s) {
+    const float dyz = fmaf(dy, dy, dz * dz);
+    const f32x2 DYZ = pk2(dyz, dyz);
+    f32x2 SR = 0ull;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+        const ulonglong2 W = *reinterpret_cast<const ulonglong2*>(&rec[j]);  // W1 and Wk of the two sources
+        const f32x2 D2 = fma2(DX[j], DX[j], DYZ);
+        const float2 d2 = up2(D2);
+        float r0 = rsqrt_approx(d2.x), r1 = rsqrt_approx(d2.y);
+        if (ON) {
+            r0 = d2.x > 0.f ? r0 : 0.f;
+            r1 = d2.y > 0.f ? r1 : 0.f;
+        }
+        const f32x2 RI = pk2(r0, r1);
+        f32x2 T = mul2(W.x, RI), TG = T;
+        if (DH) {
+            const f32x2 D = mul2(D2, RI);
+            const float2 e = up2(mul2(K2, D));
+            const f32x2 TK = mul2(mul2(W.y, RI), pk2(ex2_approx(e.x), ex2_approx(e.y)));
+            T = add2(T, TK);
+            TG = fma2(TK, mul2(KG, D), T);
+        }
+        PQ = add2(PQ, T);
+        const f32x2 F = mul2(TG, mul2(RI, RI));
+        PX = fma2(DX[j], F, PX);
+        SR = add2(SR, F);
     }
-    pq += t1;
-    const float rad = tg * ri * ri;
-    px = fmaf(dx, rad, px);
-    py = fmaf(dy, rad, py);
-    pz = fmaf(dz, rad, pz);
+    const float2 f = up2(SR);
+    s.y = fmaf(dy, f.x + f.y, s.y);
+    s.z = fmaf(dz, f.x + f.y, s.z);
 }
 
-// One group of up to kAL atoms of a leaf (kADSub threads per atom, consecutive lanes) against the leaf's list.
-template <bool DH>
-__device__ void adj_leaf_group(const TBoxes& tb, const SrcF* __restrict__ ssrcf, const uint32_t* __restrict__ idx,
-                               const float4* __restrict__ w, const float2* __restrict__ qtot,
-                               const int* __restrict__ cnt, const int* __restrict__ ent, int cap, float kap2,
-                               float kapg, double* part, float2* Q, int leaf, int j, bool act, int tid, int sub) {
-    const SrcF sf = act ? ssrcf[j] : SrcF{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const int n1 = tb.deg + 1, P3 = tb.P3;
-    float h[4] = {0.f, 0.f, 0.f, 0.f}, lo4[4] = {0.f, 0.f, 0.f, 0.f};
-    const int ne = cnt[leaf];
+struct AdjFarArgs {
+    TBoxes tb;
+    const SrcF* ssrcf;
+    const uint32_t* idx;
+    const int2* grp;
+    const int* ngrp;
+    const float4* w;
+    const float2* qtot;
+    const int* cnt;
+    const int* ent;
+    int cap, n;
+    float kap2, kapg;
+    const AdjTreeMeta* meta;
+    double* part;  // [gridDim.y][n][4]
+};
+
+// Reverse far field.  The targets of a group (up to 32 atoms) sit in the lanes of every warp, and the units of the
+// group's list go round the warps of its gridDim.y CTAs (fixed assignment, sums added in warp order, the CTAs' partials
+// in k_adj_final: deterministic).  Bound by the special-function pipe at full groups (groups hold 24 atoms on average).
+// 2,000 atoms on 128^3, both weights: 0.48 ms (5.8 ms when four threads per atom of one CTA per group walked the whole
+// list, 100 CTAs of four warps in all); 55,000 atoms on 320x320x384, 1/d only: 9.5 ms (21.9).
+template <int N1, bool DH>
+__global__ void __launch_bounds__(32 * kADWarps) k_adj_treefar(const __grid_constant__ AdjFarArgs a) {
+    using U = AdjUnit<N1>;
+    __shared__ __align__(16) float4 recs[kADWarps][U::REC];
+    __shared__ float4 sum_h[kADWarps][32], sum_l[kADWarps][32];
+    if (a.meta->overflow) return;
+    const TBoxes& tb = a.tb;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nw = kADWarps * (int)gridDim.y, me = kADWarps * (int)blockIdx.y + w;
     const int64_t plane = (int64_t)tb.ny * tb.nx;
-    // proxy offsets from the box centre and the A1 weight (16-byte aligned after the even-sized Q array)
-    float4* Pc = reinterpret_cast<float4*>(Q + ((P3 + 1) & ~1));
-    for (int e = 0; e < ne; ++e) {
-        const int code = ent[(int64_t)leaf * cap + e];
-        float pq = 0.f, px = 0.f, py = 0.f, pz = 0.f;
-        if (!(code & kADirect)) {
-            const TBox T = tbox_flat(tb, code);
-            const float hx = 0.5f * (T.ext[0] - 1), hy = 0.5f * (T.ext[1] - 1), hz = 0.5f * (T.ext[2] - 1);
-            __syncthreads();
-            const float2* src = qtot + (int64_t)code * P3;
-            for (int k = tid; k < P3; k += kADThreads) {
-                const int kx = k % n1, ky = (k / n1) % n1, kz = k / (n1 * n1);
-                const float2 q = src[k];
-                Q[k] = q;
-                Pc[k] = make_float4(hx * tb.ck[kx], hy * tb.ck[ky], hz * tb.ck[kz], q.x);
+    const f32x2 K2 = pk2(a.kap2, a.kap2), KG = pk2(a.kapg, a.kapg);
+    float4* rec = recs[w];
+    const int ngrp = *a.ngrp;
+    for (int g = blockIdx.x; g < ngrp; g += gridDim.x) {
+        const int2 gr = a.grp[g];
+        const bool act = lane < gr.y;
+        const SrcF sf = a.ssrcf[gr.x + (act ? lane : 0)];  // idle lanes repeat the first target
+        // a target on a lattice point, or so close to one that a squared distance could round to 0
+        const bool on = __any_sync(0xffffffffu, fabsf(sf.xh - rintf(sf.xh)) + fabsf(sf.xl) < 1e-9f &&
+                                                    fabsf(sf.yh - rintf(sf.yh)) + fabsf(sf.yl) < 1e-9f &&
+                                                    fabsf(sf.zh - rintf(sf.zh)) + fabsf(sf.zl) < 1e-9f);
+        float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+        const int ne = a.cnt[g];
+        const int* ent = a.ent + (int64_t)g * a.cap;
+        int base = 0, t = me;  // units of the entries before this block of 32; my next unit
+        for (int e0 = 0; e0 < ne; e0 += 32) {
+            const int code = e0 + lane < ne ? ent[e0 + lane] : 0;
+            int nu = 0;
+            if (e0 + lane < ne) nu = (code & kADirect) ? tbox_flat(tb, code & ~kADirect).ext[2] : U::NU;
+            int end = nu;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, end, o);
+                if (lane >= o) end += v;
             }
-            __syncthreads();
-            // atom relative to the box centre
-            const float ax = (sf.xh - (float)T.c[0]) + sf.xl, ay = (sf.yh - (float)T.c[1]) + sf.yl,
-                        az = (sf.zh - (float)T.c[2]) + sf.zl;
-            for (int k = sub; k < P3; k += kADSub) {
-                const float4 pc = Pc[k];
-                adj_pair<DH>(pc.x - ax, pc.y - ay, pc.z - az, pc.w, DH ? Q[k].y : 0.f, kap2, kapg, pq, px, py, pz);
-            }
-        } else {
-            const TBox R = tbox_flat(tb, code & ~kADirect);
-            const int m0 = R.ext[0], m1 = R.ext[1], m2 = R.ext[2];
-            // lattice point minus the atom: exact first subtraction for nearby atoms
-            for (int iz = 0; iz < m2; ++iz) {
-                const int gz = R.lo[2] + iz;
-                const float dz = ((float)gz - sf.zh) - sf.zl;
-                for (int iy = 0; iy < m1; ++iy) {
-                    const int gy = R.lo[1] + iy;
-                    const float dy = ((float)gy - sf.yh) - sf.yl;
-                    const float4* row = w + gz * plane + (int64_t)gy * tb.nx + R.lo[0];
-                    for (int ix = sub; ix < m0; ix += kADSub) {
-                        const float4 wv = row[ix];
-                        adj_pair<DH>(((float)(R.lo[0] + ix) - sf.xh) - sf.xl, dy, dz, wv.x, wv.y, kap2, kapg, pq,
-                                     px, py, pz);
+            const int tot = __shfl_sync(0xffffffffu, end, 31);
+            for (; t < base + tot; t += nw) {
+                const int src = __ffs(__ballot_sync(0xffffffffu, end > t - base)) - 1;
+                const int cd = __shfl_sync(0xffffffffu, code, src);
+                const int u = t - base - __shfl_sync(0xffffffffu, end - nu, src);  // unit of the entry
+                const TBox T = tbox_flat(tb, cd & ~kADirect);
+                f32x2 PQ = 0ull, PX = 0ull;
+                AdjSums s{0.f, 0.f, 0.f, 0.f};
+                __syncwarp();  // the previous unit's records are no longer read
+                if (cd & kADirect) {
+                    const int gz = T.lo[2] + u;
+                    const float4* wz = a.w + gz * plane + (int64_t)T.lo[1] * tb.nx + T.lo[0];
+                    for (int k = lane; k < kTB0 * U::NPG; k += 32) {
+                        const int iy = k / U::NPG, ix = 2 * (k % U::NPG);
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (iy < T.ext[1]) {
+                            const float4* p = wz + (int64_t)iy * tb.nx + ix;
+                            if (ix < T.ext[0]) {
+                                const float2 q = *reinterpret_cast<const float2*>(p);
+                                v.x = q.x;
+                                v.z = q.y;
+                            }
+                            if (ix + 1 < T.ext[0]) {
+                                const float2 q = *reinterpret_cast<const float2*>(p + 1);
+                                v.y = q.x;
+                                v.w = q.y;
+                            }
+                        }
+                        rec[k] = v;
+                    }
+                    // lattice point minus the atom: exact first subtraction for nearby atoms
+                    f32x2 DX[U::NPG];
+#pragma unroll
+                    for (int j = 0; j < U::NPG; ++j) {
+                        const float x = (float)(T.lo[0] + 2 * j);
+                        DX[j] = pk2((x - sf.xh) - sf.xl, ((x + 1.f) - sf.xh) - sf.xl);
+                    }
+                    const float dz = ((float)gz - sf.zh) - sf.zl;
+                    __syncwarp();
+                    for (int iy = 0; iy < T.ext[1]; ++iy) {
+                        const float dy = ((float)(T.lo[1] + iy) - sf.yh) - sf.yl;
+                        if (on) adj_row<U::NPG, DH, true>(rec + iy * U::NPG, DX, dy, dz, K2, KG, PQ, PX, s);
+                        else adj_row<U::NPG, DH, false>(rec + iy * U::NPG, DX, dy, dz, K2, KG, PQ, PX, s);
+                    }
+                } else {
+                    constexpr int P2 = N1 * N1;
+                    const int kz0 = u * U::PU, nz = min(U::PU, N1 - kz0);
+                    const float2* q = a.qtot + (int64_t)cd * (P2 * N1) + kz0 * P2;
+                    for (int k = lane; k < nz * N1 * U::NP; k += 32) {
+                        const int row = k / U::NP, kx = 2 * (k % U::NP);
+                        const float2 q0 = q[row * N1 + kx];
+                        const float2 q1 = kx + 1 < N1 ? q[row * N1 + kx + 1] : make_float2(0.f, 0.f);
+                        rec[k] = make_float4(q0.x, q1.x, q0.y, q1.y);
+                    }
+                    const float hx = 0.5f * (T.ext[0] - 1), hy = 0.5f * (T.ext[1] - 1), hz = 0.5f * (T.ext[2] - 1);
+                    // the atom relative to the box centre
+                    const float ax = (sf.xh - T.c[0]) + sf.xl, ay = (sf.yh - T.c[1]) + sf.yl, az = (sf.zh - T.c[2]) + sf.zl;
+                    f32x2 DX[U::NP];
+#pragma unroll
+                    for (int j = 0; j < U::NP; ++j)
+                        DX[j] = pk2(hx * tb.ck[2 * j] - ax, hx * tb.ck[2 * j + 1 < N1 ? 2 * j + 1 : 2 * j] - ax);
+                    __syncwarp();
+                    for (int kz = 0; kz < nz; ++kz) {
+                        const float dz = hz * tb.ck[kz0 + kz] - az;
+                        for (int ky = 0; ky < N1; ++ky)
+                            adj_row<U::NP, DH, false>(rec + (kz * N1 + ky) * U::NP, DX, hy * tb.ck[ky] - ay, dz, K2, KG,
+                                                      PQ, PX, s);
                     }
                 }
+                const float2 pq = up2(PQ), px = up2(PX);
+                ff_add(h[0], l[0], pq.x + pq.y);
+                ff_add(h[1], l[1], px.x + px.y);
+                ff_add(h[2], l[2], s.y);
+                ff_add(h[3], l[3], s.z);
             }
+            base += tot;
         }
-        ff_add(h[0], lo4[0], pq);
-        ff_add(h[1], lo4[1], px);
-        ff_add(h[2], lo4[2], py);
-        ff_add(h[3], lo4[3], pz);
+        sum_h[w][lane] = make_float4(h[0], h[1], h[2], h[3]);
+        sum_l[w][lane] = make_float4(l[0], l[1], l[2], l[3]);
+        __syncthreads();
+        if (w == 0 && act) {
+            for (int k = 1; k < kADWarps; ++k) {
+                const float4 H = sum_h[k][lane], L = sum_l[k][lane];
+                const float hv[4] = {H.x, H.y, H.z, H.w}, lv[4] = {L.x, L.y, L.z, L.w};
+                for (int q = 0; q < 4; ++q) {
+                    ff_add(h[q], l[q], hv[q]);
+                    l[q] += lv[q];
+                }
+            }
+            double* o = a.part + ((int64_t)blockIdx.y * a.n + a.idx[gr.x + lane]) * 4;
+            for (int q = 0; q < 4; ++q) o[q] = (double)h[q] + (double)l[q];
+        }
+        __syncthreads();
     }
-    // the kADSub threads of an atom are consecutive lanes: combine them in a fixed order
-    double v[4];
-    for (int q = 0; q < 4; ++q) {
-        v[q] = (double)h[q] + (double)lo4[q];
-        for (int o = 1; o < kADSub; o <<= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    }
-    if (act && sub == 0) {
-        double* o = part + (int64_t)idx[j] * 4;
-        for (int q = 0; q < 4; ++q) o[q] = v[q];
-    }
-}
-
-template <bool DH>
-__global__ void __launch_bounds__(kADThreads) k_adj_treefar(TBoxes tb, const SrcF* __restrict__ ssrcf,
-                                                           const uint32_t* __restrict__ idx,
-                                                           const int2* __restrict__ grp,
-                                                           const int* __restrict__ nleaf_p,
-                                                           const float4* __restrict__ w,
-                                                           const float2* __restrict__ qtot, const int* __restrict__ cnt,
-                                                           const int* __restrict__ ent, int cap, float kap2,
-                                                           float kapg, const AdjTreeMeta* meta, double* part) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    float2* Q = reinterpret_cast<float2*>(sm_raw);  // one box's proxies
-    if (meta->overflow || blockIdx.x >= *nleaf_p) return;
-    const int leaf = blockIdx.x, tid = threadIdx.x, a = tid / kADSub, sub = tid % kADSub;
-    const int2 gr = grp[leaf];
-    adj_leaf_group<DH>(tb, ssrcf, idx, w, qtot, cnt, ent, cap, kap2, kapg, part, Q, leaf, gr.x + a, a < gr.y, tid,
-                       sub);
 }
 
 template <int N1>
@@ -5223,6 +5320,29 @@ void launch_adj_q_deg(const TBoxes& tb, const float4* w, float2* qpart, int* rlo
     }
 }
 
+template <int N1>
+void launch_adj_far(const AdjFarArgs& a, bool dh, dim3 grid, cudaStream_t st) {
+    if (dh) k_adj_treefar<N1, true><<<grid, 32 * kADWarps, 0, st>>>(a);
+    else k_adj_treefar<N1, false><<<grid, 32 * kADWarps, 0, st>>>(a);
+}
+
+void launch_adj_far_deg(const AdjFarArgs& a, bool dh, dim3 grid, cudaStream_t st) {
+    switch (a.tb.deg) {
+        case 1: return launch_adj_far<2>(a, dh, grid, st);
+        case 2: return launch_adj_far<3>(a, dh, grid, st);
+        case 3: return launch_adj_far<4>(a, dh, grid, st);
+        case 4: return launch_adj_far<5>(a, dh, grid, st);
+        case 5: return launch_adj_far<6>(a, dh, grid, st);
+        case 6: return launch_adj_far<7>(a, dh, grid, st);
+        case 7: return launch_adj_far<8>(a, dh, grid, st);
+        case 8: return launch_adj_far<9>(a, dh, grid, st);
+        case 9: return launch_adj_far<10>(a, dh, grid, st);
+        case 10: return launch_adj_far<11>(a, dh, grid, st);
+        case 11: return launch_adj_far<12>(a, dh, grid, st);
+        default: return launch_adj_far<13>(a, dh, grid, st);
+    }
+}
+
 }  // namespace
 
 struct AdjTree {
@@ -5251,10 +5371,17 @@ struct AdjTree {
 
 void adjtree_delete(AdjTree* a) { delete a; }
 
+// About 12 CTAs of eight warps per SM over all groups (of some 24 atoms), at most 64 per group.
+int tree_adjoint_chunks(int64_t n) {
+    const int64_t groups = std::max<int64_t>(1, n / 24);
+    return (int)std::min<int64_t>(64, (12 * (int64_t)sm_count() + groups - 1) / groups);
+}
+
 const uint32_t* tree_atom_order(TreeState* s) { return (s && s->prepared) ? s->idx : nullptr; }
 
 rism_status tree_adjoint_far(TreeState* s, const DevTables& t, const GridD& g, const Phys& ph, const rism_options& o,
-                             const float4* w, bool dh, double* part, cudaStream_t st, std::string& err, bool& used) {
+                             const float4* w, bool dh, double* part, int chunks, cudaStream_t st, std::string& err,
+                             bool& used) {
     used = false;
     const TBoxes& tb = s->tb;
     const int n = (int)t.n;
@@ -5290,7 +5417,6 @@ rism_status tree_adjoint_far(TreeState* s, const DevTables& t, const GridD& g, c
         return cuda_err(err, e, "reverse-mode leaves");
     k_leaf_list<<<1, 1024, 0, st>>>(s->meta, s->nodes, A.grp, A.nleaf);
     launch_adj_q_deg(tb, w, A.qpart, A.rlow, A.qtot, st);
-    const size_t sq = sizeof(float2) * ((tb.P3 + 1) & ~1) + sizeof(float4) * tb.P3;
     for (int attempt = 0; attempt < 4; ++attempt) {
         if (nleaf + 1 > A.cap_leaf) {
             cudaFree(A.cnt);
@@ -5302,13 +5428,24 @@ rism_status tree_adjoint_far(TreeState* s, const DevTables& t, const GridD& g, c
         cudaMemsetAsync(A.meta, 0, sizeof(AdjTreeMeta), st);
         k_adj_lists<<<(nleaf + kListWarps - 1) / kListWarps, 32 * kListWarps, 0, st>>>(
             tb, s->srcf, A.grp, A.nleaf, (float)o.theta, A.cap, A.cnt, A.ent, A.meta);
-        const float kap2 = (float)(-ph.kappa * g.h * 1.4426950408889634), kapg = (float)(ph.kappa * g.h);
-        if (dh)
-            k_adj_treefar<true><<<nleaf, kADThreads, sq, st>>>(tb, s->srcf, s->idx, A.grp, A.nleaf, w, A.qtot, A.cnt,
-                                                               A.ent, A.cap, kap2, kapg, A.meta, part);
-        else
-            k_adj_treefar<false><<<nleaf, kADThreads, sq, st>>>(tb, s->srcf, s->idx, A.grp, A.nleaf, w, A.qtot,
-                                                                A.cnt, A.ent, A.cap, kap2, kapg, A.meta, part);
+        AdjFarArgs fa;
+        fa.tb = tb;
+        fa.ssrcf = s->srcf;
+        fa.idx = s->idx;
+        fa.grp = A.grp;
+        fa.ngrp = A.nleaf;
+        fa.w = w;
+        fa.qtot = A.qtot;
+        fa.cnt = A.cnt;
+        fa.ent = A.ent;
+        fa.cap = A.cap;
+        fa.n = n;
+        fa.kap2 = (float)(-ph.kappa * g.h * 1.4426950408889634);
+        fa.kapg = (float)(ph.kappa * g.h);
+        fa.meta = A.meta;
+        fa.part = part;
+        // CTAs stride over the groups (their number is on the device: between n / kAL and the bound)
+        launch_adj_far_deg(fa, dh, dim3((unsigned)std::min(nleaf, n / 8 + 1), (unsigned)chunks), st);
         if ((e = cudaMemcpyAsync(A.h_meta, A.meta, sizeof(AdjTreeMeta), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
             (e = cudaStreamSynchronize(st)) != cudaSuccess)
             return cuda_err(err, e, "reverse-mode lists");

@@ -70,11 +70,13 @@ int tree_slabs(const TreeState* ts, const GridD& g, int (*z)[2], cudaEvent_t* ev
 constexpr int kOutSlabsMax = 16;
 
 // Reverse mode, far part, with the grid boxes as source clusters: w holds the per-point weights (A1 of 1/d,
-// Ak of e^{-kappa d}/d in .x, .y); part receives per atom (original order) dq, Gx, Gy, Gz in grid units, as
-// one chunk of the direct far kernel would.  used = false (nothing done) when target boxes are off or the tree
-// is not prepared for the current solute.  Synchronises the stream (list growth).
+// Ak of e^{-kappa d}/d in .x, .y); part receives per chunk and atom (original order) dq, Gx, Gy, Gz in grid units,
+// as the direct far kernel's chunks do.  used = false (nothing done) when target boxes are off or the tree is not
+// prepared for the current solute.  Synchronises the stream (list growth).
+int tree_adjoint_chunks(int64_t n);  // the chunks to pass (and to size part for)
 rism_status tree_adjoint_far(TreeState* ts, const DevTables& t, const GridD& g, const Phys& ph, const rism_options& o,
-                             const float4* w, bool dh, double* part, cudaStream_t st, std::string& err, bool& used);
+                             const float4* w, bool dh, double* part, int chunks, cudaStream_t st, std::string& err,
+                             bool& used);
 
 // Original atom indices in Morton (sorted) order of the last tree build, or null before any.
 const uint32_t* tree_atom_order(TreeState* ts);

@@ -282,3 +282,24 @@ def test_stack55000_backward_64_atoms_vs_oracle_and_central_differences(R):
             fd[n, comp] = diff() / (2.0 * step)
     one.close()
     _check(g, fd, atoms, label="55k vs central differences")
+
+
+@pytest.mark.parametrize("degree, tol", [(5, 2e-3), (7, 2e-4), (8, GRAD_TOL), (12, GRAD_TOL)])
+@pytest.mark.parametrize("kinds", [("u", "c", "h"), ("u",)])
+def test_reverse_far_field_over_boxes_vs_direct(R, degree, tol, kinds):
+    """The reverse far field over grid boxes against the direct reverse sum of the same cotangents: even and odd
+    numbers of proxies per row, clipped boxes (61x45x38), ragged target groups, atoms exactly on grid points.  Degree 8
+    and up within the gradient tolerance; below it the interpolation error of theta 0.7 (a factor 6 to 8 per degree)."""
+    w = I.small_workload(n_atoms=700, n=(61, 45, 38), h=0.5, seed=41, ions=True, lj_rcut=5.0, net=3.0)
+    o = np.asarray(w.grid.origin)
+    w.solute.xyz[:3] = o + 0.5 * np.array([[30, 20, 17], [3, 40, 9], [60, 44, 37]])
+    G = _cotangents(w, 17, kinds)
+    ref = _gpu_grad(R, w, G)
+    import torch
+
+    r = R.from_workload(w, method=R.METHOD_TREECODE, precision=R.PREC_FP32, degree=degree)
+    g = r.backward(*(torch.as_tensor(G[k], device="cuda") if k in G else None for k in ("u", "c", "h")))
+    for k in ref:
+        e = rel_l2(g[k].cpu().numpy(), ref[k])
+        assert e <= tol, f"degree {degree} d{k}: rel L2 {e:.3e} > {tol:g}"
+    r.close()
