@@ -303,3 +303,33 @@ def test_reverse_far_field_over_boxes_vs_direct(R, degree, tol, kinds):
         e = rel_l2(g[k].cpu().numpy(), ref[k])
         assert e <= tol, f"degree {degree} d{k}: rel L2 {e:.3e} > {tol:g}"
     r.close()
+
+
+@pytest.mark.parametrize("mode", ["none", "rcut", "tol"])
+@pytest.mark.parametrize("n, sites", [(70, ["O"]), (70, ["O", "H", "Na+", "Cl-", "O", "H"]), (2600, ["O", "H", "Na+"]),
+                                      (10000, ["O", "H", "Na+", "Cl-"])])
+def test_near_columns_vs_oracle(R, mode, n, sites):
+    """The near part of the reverse mode over its column tiles: one to six sites, each LJ cut-off mode, eight down to
+    one warp per atom, a solute larger than the grid (atoms outside it), an atom on a grid point, every atom or 24
+    sampled ones (that one included) against the oracle.  A cotangent that is not a number beyond every cut-off of an
+    atom leaves that atom's LJ gradients alone."""
+    import torch
+
+    w = I.small_workload(n_atoms=n, n=(27, 19, 22), h=0.5, seed=61, lj_rcut=4.0 if mode == "rcut" else 0.0, net=1.0)
+    if mode == "tol":
+        w.opts["lj_tol"] = 1e-2
+    w.solvent = I.solvent(sites)
+    w.solute.xyz[5] = np.asarray(w.grid.origin) + 0.5 * np.array([11, 7, 13])
+    G = _cotangents(w, 23, ("u", "c", "h") if "Na+" in sites else ("u", "c"))
+    p = O.Problem.from_workload(w)
+    atoms = np.arange(n) if n < 100 else np.union1d([5], np.random.default_rng(3).choice(n, 24, replace=False))
+    g = _gpu_grad(R, w, G)
+    _check(g, O.grad(p, atoms, G["u"], G["c"], G.get("h")), atoms, label=f"{mode} {n} atoms, {len(sites)} sites")
+    if mode == "rcut":
+        d = np.linalg.norm(w.solute.xyz - (np.asarray(w.grid.origin) + 0.5 * np.array([26, 18, 21])), axis=1)
+        far = d > 4.5
+        G["u"] = G["u"].copy()
+        G["u"][:, 21, 18, 26] = np.nan
+        b = _gpu_grad(R, w, G)
+        for k in ("sigma", "eps"):
+            assert np.array_equal(b[k][far], g[k][far]) and np.isnan(b[k][d < 3.5]).all()
