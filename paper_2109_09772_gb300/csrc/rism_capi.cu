@@ -71,7 +71,10 @@ struct rism_ctx {
     double2* d_lra_atom = nullptr;
     int64_t lra_atom_cap = 0;
     double* d_lra_tot = nullptr;
+    size_t lra_tot_len = 0;
     double* h_lra_tot = nullptr;  // pinned [3]
+    float* d_lra_tab = nullptr;   // cubic pieces of the overlap integrals for lra_tab_key = (eta, kappa)
+    double lra_tab_key[2] = {0.0, -1.0};
     // the atoms in a spatial order for the pair sum (position -> original index), recomputed for a new solute
     int* h_lra_perm = nullptr;    // pinned [lra_perm_cap]
     int* d_lra_perm = nullptr;
@@ -653,7 +656,7 @@ void lra_order(const double* raw, int64_t n, int* perm) {
         ext[d] = std::max(hi[d] - lo[d], 1e-6);
         vol *= ext[d];
     }
-    const double side = std::cbrt(vol / (double)std::max<int64_t>(1, n / 32));
+    const double side = std::cbrt(vol / (double)std::max<int64_t>(1, n / 32)), iside = 1.0 / side;
     int nc[3];
     for (int d = 0; d < 3; ++d) nc[d] = std::max(1, std::min(1024, (int)std::ceil(ext[d] / side)));
     const int64_t ncell = (int64_t)nc[0] * nc[1] * nc[2];
@@ -672,7 +675,7 @@ void lra_order(const double* raw, int64_t n, int* perm) {
     for (int64_t i = 0; i < n; ++i) {
         int cc[3];
         for (int d = 0; d < 3; ++d)
-            cc[d] = std::min(nc[d] - 1, std::max(0, (int)((raw[6 * i + d] - lo[d]) / side)));
+            cc[d] = std::min(nc[d] - 1, (int)((raw[6 * i + d] - lo[d]) * iside));  // never negative
         cell[(size_t)i] = rank[(size_t)(((int64_t)cc[2] * nc[1] + cc[1]) * nc[0] + cc[0])];
         ++start[(size_t)cell[(size_t)i] + 1];
     }
@@ -724,10 +727,26 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
             return cuda_fail(c, e, "LRA atom sums");
         c->lra_atom_cap = n;
     }
-    if (!c->d_lra_tot) {
-        if ((e = cudaMalloc(&c->d_lra_tot, sizeof(double) * 3)) != cudaSuccess ||
-            (e = cudaMallocHost(&c->h_lra_tot, sizeof(double) * 3)) != cudaSuccess)
+    if (lra_total_doubles(n) != c->lra_tot_len) {  // the counter's place depends on the length
+        cudaFree(c->d_lra_tot);
+        c->d_lra_tot = nullptr;
+        c->lra_tot_len = 0;
+        const size_t len = lra_total_doubles(n);
+        if ((!c->h_lra_tot && (e = cudaMallocHost(&c->h_lra_tot, sizeof(double) * 3)) != cudaSuccess) ||
+            (e = cudaMalloc(&c->d_lra_tot, sizeof(double) * len)) != cudaSuccess ||
+            (e = cudaMemsetAsync(c->d_lra_tot, 0, sizeof(double) * len, c->st)) != cudaSuccess)
             return cuda_fail(c, e, "LRA totals");
+        c->lra_tot_len = len;
+    }
+    if (!c->d_lra_tab || c->lra_tab_key[0] != c->ph.eta || c->lra_tab_key[1] != c->ph.kappa) {
+        if (!c->d_lra_tab && (e = cudaMalloc(&c->d_lra_tab, sizeof(float) * 8 * kLraTab)) != cudaSuccess)
+            return cuda_fail(c, e, "LRA kernel table");
+        std::vector<float> tab(8 * kLraTab);
+        lra_table(c->ph, tab.data());
+        if ((e = cudaMemcpy(c->d_lra_tab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+            return cuda_fail(c, e, "LRA kernel table");
+        c->lra_tab_key[0] = c->ph.eta;
+        c->lra_tab_key[1] = c->ph.kappa;
     }
     if (n > c->lra_perm_cap) {
         cudaFree(c->d_lra_perm);
@@ -751,7 +770,7 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
             return cuda_fail(c, e, "LRA atom order upload");
         c->lra_perm_version = c->solute_version;
     }
-    if ((e = launch_lra(c->t, c->gd, c->ph, sms, c->d_lra_perm, static_cast<SrcF*>(c->d_lra_src), c->d_lra_part,
+    if ((e = launch_lra(c->t, c->gd, c->ph, sms, c->d_lra_perm, static_cast<SrcF*>(c->d_lra_src), c->d_lra_tab, c->d_lra_part,
                         c->d_lra_atom, c->d_lra_tot, c->o.wait_limit, c->st)) != cudaSuccess)
         return cuda_fail(c, e, "LRA kernels");
     if ((e = cudaMemcpyAsync(c->h_lra_tot, c->d_lra_tot, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->st)) !=
@@ -768,7 +787,7 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
         const double theta = (Q * c->qs[k] > 0.0) ? 1.0 : 0.0;
         T[k] = 0.5 * theta * A * A * Shh - 0.5 * A * B * Shc;
     }
-    c->info.launches = 4;
+    c->info.launches = 3;
     return RISM_OK;
 }
 
@@ -893,6 +912,7 @@ void rism_destroy(rism_ctx* c) {
     cudaFree(c->d_lra_src);
     cudaFreeHost(c->h_lra_perm);
     cudaFree(c->d_lra_tot);
+    cudaFree(c->d_lra_tab);
     cudaFreeHost(c->h_lra_tot);
     cudaFree(c->d_ktab);
     cudaFree(c->d_kstage[0]);

@@ -92,3 +92,42 @@ def test_edge_cases(R):
     r.set_solute(np.zeros((0, 3)), [], [], [])
     assert np.all(r.lra_integral() == 0.0)
     r.close()
+
+
+@pytest.mark.parametrize("kappa", [0.03, 0.5])
+def test_pair_tables_against_closed_forms(R, kappa):
+    """Two charges of one sign at 40 distances from 0.05 A to beyond the short-range radius (8.485 A), its two sides
+    included, on one context whose screening constant differs from the test before (the cubic pieces are rebuilt):
+    the atoms' sums are I(0) + I(R), no term cancels."""
+    R_ = np.concatenate([np.linspace(0.05, 8.4, 30), np.sqrt(72.0) * (1.0 + np.array([-1e-3, -1e-5, 1e-5, 1e-3])),
+                         [9.0, 12.0, 20.0, 40.0, 80.0, 160.0]])
+    sol = I.solvent(["O", "H", "Na+", "Cl-"])
+    r = R.Rism((20, 20, 20), 0.5, (0.0, 0.0, 0.0), kappa=kappa, method=R.METHOD_DIRECT, precision=R.PREC_FP32)
+    r.set_solvent(sol.q, sol.sigma, sol.eps, sol.rho, sol.is_ion)
+    hc, hh = O.lra_pair(1.0, kappa, np.concatenate([[0.0], R_]))
+    for k, d in enumerate(R_):
+        xyz = np.array([[1.3, 2.1, 0.7], [1.3, 2.1, 0.7]])
+        xyz[1] += d * np.array([2.0, -3.0, 6.0]) / 7.0
+        r.set_solute(xyz, [1.0, 1.0], [1.0, 1.0], [0.1, 0.1])
+        _, a = r.lra_integral(atom_sums=True)
+        ref = np.tile([[hc[0] + hc[k + 1], hh[0] + hh[k + 1]]], (2, 1))
+        _check_atoms(a.cpu().numpy(), ref, f"R = {d}")
+    r.close()
+
+
+@pytest.mark.parametrize("n", [1, 63, 65, 129, 700])
+def test_target_groups_tiles_and_totals(R, n):
+    """Source tiles, target groups and the CTAs of the totals at their edges, solutes of different size one after
+    another on one context, charges of one sign (no cancellation): every atom's sums and T."""
+    w = I.small_workload(n_atoms=n, n=(20, 20, 20), h=0.5, seed=51, ions=True, lj_rcut=4.0, net=1.0)
+    q = 0.1 + np.abs(w.solute.q)
+    r = R.from_workload(w, method=R.METHOD_TREECODE, precision=R.PREC_FP32)
+    for m in (n, max(1, n // 2), n):
+        s = w.solute
+        part = I.Workload(w.name, I.Solute(s.xyz[:m], q[:m], s.sigma[:m], s.eps[:m]), w.solvent, w.grid, w.opts)
+        r.set_solute(s.xyz[:m], q[:m], s.sigma[:m], s.eps[:m])
+        T, a = r.lra_integral(atom_sums=True)
+        p = O.Problem.from_workload(part)
+        _check_atoms(a.cpu().numpy(), O.lra_atom_sums(p, np.arange(m)), f"{m} atoms")
+        assert rel_l2(T, O.lra_integral(p)[0]) <= TOL
+    r.close()
