@@ -46,6 +46,8 @@ struct rism_ctx {
     DevErr* d_err = nullptr;
     DevErr* h_err = nullptr;  // pinned
     double* d_tail = nullptr;
+    float4* d_sr = nullptr;  // short-range pieces of the FP32 direct sum, built for sr_key
+    double sr_key[4] = {0.0, 0.0, 0.0, -1.0};
     // the solute, [n][6] x, y, z, q, sigma, eps, in page-locked host memory: uploaded as it stands (by the
     // replayed graph's copy node or an asynchronous copy); every entry point that uploads it synchronises its
     // stream before it returns, so rism_set_solute never overwrites it under a copy of a completed call
@@ -168,6 +170,20 @@ rism_status reserve_tables(rism_ctx* c) {
     c->t.err = c->d_err;
     c->gd = GridD{c->g.nx, c->g.ny, c->g.nz, c->g.h, c->g.origin[0], c->g.origin[1], c->g.origin[2]};
     make_phys(c);
+    if (c->o.method == RISM_METHOD_DIRECT && c->o.precision == RISM_PREC_FP32) {
+        const double key[4] = {c->ph.eta, c->gd.h, c->ph.a, c->ph.rs};
+        if (!c->d_sr || std::memcmp(key, c->sr_key, sizeof key) != 0) {
+            if (!c->d_sr && (e = cudaMalloc(&c->d_sr, sizeof(float4) * 2 * kNTab)) != cudaSuccess)
+                return cuda_fail(c, e, "short-range table");
+            std::vector<float4> tab(2 * kNTab);
+            short_range_table(c->ph, c->gd.h, tab.data());
+            if ((e = cudaMemcpy(c->d_sr, tab.data(), sizeof(float4) * tab.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+                return cuda_fail(c, e, "short-range table");
+            std::memcpy(c->sr_key, key, sizeof key);
+        }
+        c->t.sr = c->d_sr;
+        c->t.sr_inv = (float)(kNTab / (c->ph.rs / c->gd.h));
+    }
     return RISM_OK;
 }
 
@@ -898,6 +914,7 @@ void rism_destroy(rism_ctx* c) {
     cudaFreeHost(c->h_tail);
     cudaFreeHost(c->h_raw);
     cudaFree(c->d_tail);
+    cudaFree(c->d_sr);
     for (int k = 0; k < 3; ++k) cudaFree(c->d_stage[k]);
     if (c->ev[0]) cudaEventDestroy(c->ev[0]);
     if (c->ev[1]) cudaEventDestroy(c->ev[1]);

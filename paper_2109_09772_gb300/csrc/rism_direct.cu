@@ -19,6 +19,7 @@
 // every thread owns a strip of P consecutive x points at one (y, z) and reads
 // each atom as a shared-memory broadcast.
 #include <cmath>
+#include <vector>
 
 #include "rism_kernels.h"
 
@@ -154,6 +155,32 @@ __global__ void __launch_bounds__(kTailThreads) k_lj_tail(const LJd* lj, int64_t
 cudaError_t launch_lj_tail(const DevTables& t, int S, double* dev_out, cudaStream_t st) {
     k_lj_tail<<<S, kTailThreads, 0, st>>>(t.ljd, t.n, t.smax, dev_out);
     return cudaGetLastError();
+}
+
+// In grid units; F_h = e^{a^2-2ax} erfc(x-a) + e^{a^2+2ax} erfc(x+a), x = d h / eta, a = kappa eta / 2, with the
+// derivatives dF_c/dx = -2/sqrt(pi) e^{-x^2} and dF_h/dx = -2a e^{a^2-2ax} erfc(x-a) + 2a e^{a^2+2ax} erfc(x+a) -
+// 4/sqrt(pi) e^{-x^2}; built in FP64.
+void short_range_table(const Phys& ph, double h, float4* tab) {
+    const double sx = h / ph.eta, a = ph.a, D = ph.rs / h / kNTab;
+    const double tsp = 2.0 / std::sqrt(3.14159265358979323846);
+    std::vector<double> fc(kNTab + 1), gc(kNTab + 1), fh(kNTab + 1), gh(kNTab + 1);
+    for (int k = 0; k <= kNTab; ++k) {
+        const double x = k * D * sx, ex = std::exp(-x * x);
+        const double em = std::exp(a * a - 2.0 * a * x), ep = std::exp(a * a + 2.0 * a * x);
+        const double cm = std::erfc(x - a), cp = std::erfc(x + a);
+        fc[k] = std::erfc(x);
+        gc[k] = -tsp * ex * sx * D;  // derivative per segment length
+        fh[k] = em * cm + ep * cp;
+        gh[k] = (-2.0 * a * em * cm + 2.0 * a * ep * cp - 2.0 * tsp * ex) * sx * D;
+    }
+    auto herm = [](double f0, double f1, double g0, double g1) {
+        return make_float4((float)f0, (float)g0, (float)(3.0 * (f1 - f0) - 2.0 * g0 - g1),
+                           (float)(2.0 * (f0 - f1) + g0 + g1));
+    };
+    for (int k = 0; k < kNTab; ++k) {
+        tab[2 * k] = herm(fc[k], fc[k + 1], gc[k], gc[k + 1]);
+        tab[2 * k + 1] = herm(fh[k], fh[k + 1], gh[k], gh[k + 1]);
+    }
 }
 
 // ------------------------------------------------------- common epilogue
@@ -305,25 +332,90 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct64(GridD g, Phys ph, const
 // grid coordinates are exact integers, so dx = (i - xh) - xl is exact to half
 // an ulp of dx for every nearby atom.  Per-tile FP32 partial sums are folded
 // into float-float totals (TwoSum), which carry ~48 bits.
-template <int SM, int P, int BX, int BY, int BZ, int T, bool DU, bool DH>
-__global__ void __launch_bounds__(BX* BY* BZ) k_direct32(GridD g, Phys ph, const SrcF* __restrict__ srcf,
-                                                          const LJf* __restrict__ lj, int64_t n, Outputs o,
-                                                          DevErr* err, long long wlim, int dbg) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    SrcF* ssrc = reinterpret_cast<SrcF*>(smem);
-    LJf* slj = reinterpret_cast<LJf*>(smem + 2 * T * sizeof(SrcF));
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * T * sizeof(SrcF) + 2 * T * SM * sizeof(LJf));
+//
+// A warp owns a block of 2P x 4 x 4 points (P consecutive x points per lane), a CTA two by two of them.  Per tile of
+// atoms a warp takes the long-range sums of all of them, two sources per instruction, and then only the atoms within
+// the short-range radius or their largest LJ cut-off of its block, listed by ballots, for the LJ terms and the erfc
+// remainders (a few in a hundred of a solute's atoms).
+constexpr int kDirectT = 64;  // atoms per tile (two ballots)
 
-    const int tid = threadIdx.x;
-    const int tx = tid % BX, ty = (tid / BX) % BY, tz = tid / (BX * BY);
-    const int i0 = (blockIdx.x * BX + tx) * P, j = blockIdx.y * BY + ty, k = blockIdx.z * BZ + tz;
+// Sources 2l and 2l + 1 of a tile, field by field (two-wide operands); an odd count is padded with a zero charge 10^6
+// grid units away, whose terms are exactly zero.
+struct DirRec {
+    float4 x;  // xh0, xh1, xl0, xl1
+    float4 y, z;
+    float4 q;  // q0, q1, 0, 0
+};
+
+// The long-range sums of one tile at P points: per pair dx = (x - x_hi) - x_lo, d2, r = rsqrt(d2), q r, and with DH
+// the screening factor by ex2.  ON: some source of the tile sits on a lattice point; d2 = 0 adds nothing here.
+template <int P, bool DH, bool ON>
+__device__ __forceinline__ void direct_far(const DirRec* rec, int np, const f32x2 (&GX)[P], f32x2 FY, f32x2 FZ, f32x2 K2,
+                                           f32x2 (&P1)[P], f32x2 (&PK)[P]) {
+#pragma unroll 2
+    for (int l = 0; l < np; ++l) {
+        const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(&rec[l].x);
+        const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(&rec[l].y);
+        const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(&rec[l].z);
+        const f32x2 Q = *reinterpret_cast<const f32x2*>(&rec[l].q);
+        const f32x2 DY = sub2(sub2(FY, Y.x), Y.y);
+        const f32x2 DZ = sub2(sub2(FZ, Z.x), Z.y);
+        const f32x2 DYZ = fma2(DY, DY, mul2(DZ, DZ));
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const f32x2 DX = sub2(sub2(GX[p], X.x), X.y);
+            const f32x2 D2 = fma2(DX, DX, DYZ);
+            const float2 d2 = up2(D2);
+            float r0 = rsqrt_approx(d2.x), r1 = rsqrt_approx(d2.y);
+            if (ON) {
+                r0 = d2.x > 0.f ? r0 : 0.f;
+                r1 = d2.y > 0.f ? r1 : 0.f;
+            }
+            const f32x2 RI = pk2(r0, r1);
+            const f32x2 QR = mul2(Q, RI);
+            P1[p] = add2(P1[p], QR);
+            if (DH) {
+                const float2 e = up2(mul2(K2, mul2(D2, RI)));
+                PK[p] = fma2(QR, pk2(ex2_approx(e.x), ex2_approx(e.y)), PK[p]);
+            }
+        }
+    }
+}
+
+// Bound by the special-function pipe (a reciprocal square root and an exponential per pair).  2,000 atoms on 128^3, 4
+// sites: 2.1 ms, of which the long-range sums are 1.25 ms at the pipe's rate; 5.8 ms when every pair also took a
+// reciprocal, its sites' cut-off tests and a divergent branch to the remainders, in scalar instructions.
+template <int SM, int P, bool DU, bool DH>
+__global__ void __launch_bounds__(128, SM > 4 ? 2 : (P > 2 ? 3 : 4))
+    k_direct32(GridD g, Phys ph, const SrcF* __restrict__ srcf, const LJf* __restrict__ lj, int64_t n,
+               const float4* __restrict__ sr, float sr_inv, Outputs o, DevErr* err, long long wlim, int dbg) {
+    constexpr int T = kDirectT;
+    extern __shared__ __align__(16) unsigned char smem[];
+    SrcF* ssrc = reinterpret_cast<SrcF*>(smem);                                   // [2][T]
+    LJf* slj = reinterpret_cast<LJf*>(smem + 2 * T * sizeof(SrcF));               // [2][T][SM]
+    DirRec* rec = reinterpret_cast<DirRec*>(slj + 2 * T * SM);                    // [T / 2]
+    uint64_t* bar = reinterpret_cast<uint64_t*>(rec + T / 2);                     // [2]
+    int* list = reinterpret_cast<int*>(bar + 2);                                   // [4][T]
+    float4* tab = reinterpret_cast<float4*>(list + 4 * T);                         // [2 kNTab]
+
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int bx = (blockIdx.x * 2 + (w & 1)) * 2 * P, by = (blockIdx.y * 2 + (w >> 1)) * 4, bz = blockIdx.z * 4;
+    const int i0 = bx + (lane & 1) * P, j = by + ((lane >> 1) & 3), k = bz + (lane >> 3);
+    f32x2 GX[P];
     float gx[P];
 #pragma unroll
-    for (int p = 0; p < P; ++p) gx[p] = (float)(i0 + p);
+    for (int p = 0; p < P; ++p) {
+        gx[p] = (float)(i0 + p);
+        GX[p] = pk2(gx[p], gx[p]);
+    }
     const float fy = (float)j, fz = (float)k;
+    const f32x2 FY = pk2(fy, fy), FZ = pk2(fz, fz);
+    const float wlo[3] = {(float)bx, (float)by, (float)bz};
+    const float whi[3] = {(float)(bx + 2 * P - 1), (float)(by + 3), (float)(bz + 3)};
     const float rs2 = (float)((ph.rs / g.h) * (ph.rs / g.h));
     const float xs = (float)(g.h / ph.eta);                            // x = d_grid * xs
     const float kap2 = (float)(-ph.kappa * g.h * 1.4426950408889634);  // e^{-kappa d} = 2^(kap2 d_grid)
+    const f32x2 K2 = pk2(kap2, kap2);
     const float a = (float)ph.a;
     const float c0h = (float)(ph.phi_c0 * g.h), h0h = (float)(ph.phi_h0 * g.h);
     const bool DC = o.c != nullptr;
@@ -338,6 +430,8 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct32(GridD g, Phys ph, const
     unsigned hit = 0u;
 
     const int ntiles = (int)((n + T - 1) / T);
+    if (sr)
+        for (int q = tid; q < 2 * kNTab; q += 128) tab[q] = sr[q];
     if (tid == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
@@ -370,60 +464,139 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct32(GridD g, Phys ph, const
         const int cnt = (int)min((int64_t)T, n - (int64_t)t * T);
         const SrcF* Sx = ssrc + st * T;
         const LJf* L = slj + st * T * SM;
-        float p1[P], pk[P], psc[P], psh[P], plj[P][SM];
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-            p1[p] = pk[p] = psc[p] = psh[p] = 0.f;
-#pragma unroll
-            for (int s = 0; s < SM; ++s) plj[p][s] = 0.f;
+        if (tid < T / 2) {  // the pair records of the tile
+            const int s0 = 2 * tid, s1 = s0 + 1;
+            float4 a0 = make_float4(1e6f, 1e6f, 1e6f, 0.f), a1 = make_float4(0.f, 0.f, 0.f, 0.f), b0 = a0, b1 = a1;
+            if (s0 < cnt) {
+                a0 = *reinterpret_cast<const float4*>(&Sx[s0].xh);
+                a1 = *reinterpret_cast<const float4*>(&Sx[s0].xl);
+            }
+            if (s1 < cnt) {
+                b0 = *reinterpret_cast<const float4*>(&Sx[s1].xh);
+                b1 = *reinterpret_cast<const float4*>(&Sx[s1].xl);
+            }
+            rec[tid].x = make_float4(a0.x, b0.x, a1.x, b1.x);
+            rec[tid].y = make_float4(a0.y, b0.y, a1.y, b1.y);
+            rec[tid].z = make_float4(a0.z, b0.z, a1.z, b1.z);
+            rec[tid].q = make_float4(a0.w, b0.w, 0.f, 0.f);
         }
-        for (int aa = 0; aa < cnt; ++aa) {
-            const float4 g0 = *reinterpret_cast<const float4*>(&Sx[aa].xh);
-            const float4 g1 = *reinterpret_cast<const float4*>(&Sx[aa].xl);
-            const float dy = (fy - g0.y) - g1.y;
-            const float dz = (fz - g0.z) - g1.z;
-            const float dyz2 = fmaf(dy, dy, dz * dz);
+        // the atoms that reach the warp's block: within r_short or the largest cut-off of their sites (0.01 grid units
+        // of slack for the position rounded to its high part)
+        auto reach = [&](int i) {
+            if (i >= cnt) return false;
+            const float4 c = *reinterpret_cast<const float4*>(&Sx[i].xh);
+            float r2 = rs2;
+            if (DU)
+#pragma unroll
+                for (int s = 0; s < SM; ++s) r2 = fmaxf(r2, L[i * SM + s].rc2);
+            const float qx = fmaxf(0.f, fmaxf(wlo[0] - c.x, c.x - whi[0]));
+            const float qy = fmaxf(0.f, fmaxf(wlo[1] - c.y, c.y - whi[1]));
+            const float qz = fmaxf(0.f, fmaxf(wlo[2] - c.z, c.z - whi[2]));
+            const float lim = sqrtf(r2) + 0.01f;
+            return fmaf(qx, qx, fmaf(qy, qy, qz * qz)) < lim * lim;
+        };
+        const bool k0 = reach(lane), k1 = reach(lane + 32);
+        const bool mine = (lane < cnt && Sx[lane].on_grid != 0.f) || (lane + 32 < cnt && Sx[lane + 32].on_grid != 0.f);
+        const bool on = __any_sync(0xffffffffu, mine);
+        const unsigned m0 = __ballot_sync(0xffffffffu, k0), m1 = __ballot_sync(0xffffffffu, k1);
+        const unsigned lt = (1u << lane) - 1u;
+        int* wl = list + w * T;
+        const int near = __popc(m0) + __popc(m1);
+        if (k0) wl[__popc(m0 & lt)] = lane;
+        if (k1) wl[__popc(m0) + __popc(m1 & lt)] = lane + 32;
+        __syncthreads();  // the records and the list
+        {
+            f32x2 P1[P], PK[P];
+#pragma unroll
+            for (int p = 0; p < P; ++p) P1[p] = PK[p] = 0ull;
+            const int np = (cnt + 1) >> 1;
+            if (on) direct_far<P, DH, true>(rec, np, GX, FY, FZ, K2, P1, PK);
+            else direct_far<P, DH, false>(rec, np, GX, FY, FZ, K2, P1, PK);
 #pragma unroll
             for (int p = 0; p < P; ++p) {
-                const float dx = (gx[p] - g0.x) - g1.x;
-                const float d2 = fmaf(dx, dx, dyz2);
-                const float rr = rsqrt_approx(d2);
-                const float ri = d2 > 0.f ? rr : 0.f;
-                const float qr = g0.w * ri;
-                p1[p] += qr;
-                if (DH) pk[p] = fmaf(qr, ex2_approx(kap2 * (d2 * ri)), pk[p]);
-                if (d2 < rs2) {
-                    if (d2 > 0.f) {
-                        const float x = d2 * ri * xs;
-                        if (DC) psc[p] = fmaf(qr, erfcf(x), psc[p]);
-                        if (DH) psh[p] = fmaf(qr, __expf(-x * x) * (erfcxf(x - a) + erfcxf(x + a)), psh[p]);
-                    } else {
-                        hit |= 1u << p;
-                        if (DC) psc[p] -= g0.w * c0h;
-                        if (DH) psh[p] -= g0.w * h0h;
-                    }
-                }
-                if (DU) {
-                    const float r2i = rcp_approx(d2);
-                    const float r6 = r2i * r2i * r2i;
-#pragma unroll
-                    for (int s = 0; s < SM; ++s) {
-                        const float4 l = *reinterpret_cast<const float4*>(&L[aa * SM + s]);
-                        if (d2 < l.z) plj[p][s] = fmaf(r6, fmaf(l.x, r6, -l.y), plj[p][s]);
-                    }
+                const float2 s1 = up2(P1[p]);
+                ff_add(f1h[p], f1l[p], s1.x + s1.y);
+                if (DH) {
+                    const float2 sk = up2(PK[p]);
+                    ff_add(fkh[p], fkl[p], sk.x + sk.y);
                 }
             }
         }
+        if (near > 0) {
+            f32x2 plj[P / 2][SM];  // two points per register pair
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-            ff_add(f1h[p], f1l[p], p1[p]);
-            if (DH) ff_add(fkh[p], fkl[p], pk[p]);
-            if (DC) ff_add(sch[p], scl[p], psc[p]);
-            if (DH) ff_add(shh[p], shl[p], psh[p]);
-            if (DU) {
+            for (int p = 0; p < P / 2; ++p)
 #pragma unroll
-                for (int s = 0; s < SM; ++s) ff_add(ljh[p][s], ljl[p][s], plj[p][s]);
+                for (int s = 0; s < SM; ++s) plj[p][s] = 0ull;
+            for (int q = 0; q < near; ++q) {
+                const int aa = wl[q];
+                const float4 g0 = *reinterpret_cast<const float4*>(&Sx[aa].xh);
+                const float4 g1 = *reinterpret_cast<const float4*>(&Sx[aa].xl);
+                const float dy = (fy - g0.y) - g1.y;
+                const float dz = (fz - g0.z) - g1.z;
+                const float dyz2 = fmaf(dy, dy, dz * dz);
+                float d2[P];
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    const float dx = (gx[p] - g0.x) - g1.x;
+                    d2[p] = fmaf(dx, dx, dyz2);
+                }
+                if (DU) {
+#pragma unroll
+                    for (int p = 0; p < P / 2; ++p) {
+                        const float r0 = rcp_approx(d2[2 * p]), r1 = rcp_approx(d2[2 * p + 1]);
+                        const float a6 = r0 * r0 * r0, b6 = r1 * r1 * r1;
+#pragma unroll
+                        for (int s = 0; s < SM; ++s) {
+                            const float4 l = *reinterpret_cast<const float4*>(&L[aa * SM + s]);
+                            // a point outside the cut-off adds +0
+                            const f32x2 R6 = pk2(d2[2 * p] < l.z ? a6 : 0.f, d2[2 * p + 1] < l.z ? b6 : 0.f);
+                            plj[p][s] = fma2(R6, fma2(pk2(l.x, l.x), R6, pk2(-l.y, -l.y)), plj[p][s]);
+                        }
+                    }
+                }
+                float dmin = d2[0];
+#pragma unroll
+                for (int p = 1; p < P; ++p) dmin = fminf(dmin, d2[p]);
+                if (dmin < rs2) {
+#pragma unroll
+                    for (int p = 0; p < P; ++p) {
+                        if (d2[p] >= rs2) continue;
+                        if (d2[p] > 0.f) {
+                            const float ri = rsqrt_approx(d2[p]), qr = g0.w * ri;
+                            if (sr) {
+                                int it;
+                                const float tt = seg_split(d2[p] * ri * sr_inv, it);
+                                if (DC) {
+                                    const float4 c = tab[2 * it];
+                                    ff_add(sch[p], scl[p], qr * fmaf(fmaf(fmaf(c.w, tt, c.z), tt, c.y), tt, c.x));
+                                }
+                                if (DH) {
+                                    const float4 c = tab[2 * it + 1];
+                                    ff_add(shh[p], shl[p], qr * fmaf(fmaf(fmaf(c.w, tt, c.z), tt, c.y), tt, c.x));
+                                }
+                            } else {
+                                const float x = d2[p] * ri * xs;
+                                if (DC) ff_add(sch[p], scl[p], qr * erfcf(x));
+                                if (DH) ff_add(shh[p], shl[p], qr * (__expf(-x * x) * (erfcxf(x - a) + erfcxf(x + a))));
+                            }
+                        } else {
+                            hit |= 1u << p;
+                            if (DC) ff_add(sch[p], scl[p], -(g0.w * c0h));
+                            if (DH) ff_add(shh[p], shl[p], -(g0.w * h0h));
+                        }
+                    }
+                }
             }
+            if (DU)
+#pragma unroll
+                for (int p = 0; p < P / 2; ++p)
+#pragma unroll
+                    for (int s = 0; s < SM; ++s) {
+                        const float2 v = up2(plj[p][s]);
+                        ff_add(ljh[2 * p][s], ljl[2 * p][s], v.x);
+                        ff_add(ljh[2 * p + 1][s], ljl[2 * p + 1][s], v.y);
+                    }
         }
         __syncthreads();
         if (tid == 0 && t + 2 < ntiles) issue(t + 2);
@@ -470,6 +643,17 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct32(GridD g, Phys ph, const
 namespace {
 constexpr int kP = 4, kBX = 8, kBY = 4, kBZ = 4, kT = 64;
 
+template <int SM, int P, bool DU, bool DH>
+cudaError_t run_direct32(const GridD& g, const Phys& ph, const DevTables& t, Outputs o, long long wl, int dbg,
+                         cudaStream_t st) {
+    const size_t sm = 2 * kDirectT * sizeof(SrcF) + 2 * kDirectT * SM * sizeof(LJf) + (kDirectT / 2) * sizeof(DirRec) +
+                      2 * sizeof(uint64_t) + 4 * kDirectT * sizeof(int) + 2 * kNTab * sizeof(float4);
+    const dim3 grid((g.nx + 4 * P - 1) / (4 * P), (g.ny + 7) / 8, (g.nz + 3) / 4);
+    raise_dyn_smem(k_direct32<SM, P, DU, DH>, sm);
+    k_direct32<SM, P, DU, DH><<<grid, 128, sm, st>>>(g, ph, t.srcf, t.ljf, t.n, t.sr, t.sr_inv, o, t.err, wl, dbg);
+    return cudaGetLastError();
+}
+
 template <int SM, bool DU, bool DH>
 cudaError_t run_direct(const GridD& g, const Phys& ph, const DevTables& t, int prec, Outputs o, long long wl,
                        int dbg, cudaStream_t st) {
@@ -481,10 +665,11 @@ cudaError_t run_direct(const GridD& g, const Phys& ph, const DevTables& t, int p
         raise_dyn_smem(kern, sm);
         kern<<<grid, block, sm, st>>>(g, ph, t.geo, t.ljd, t.n, o, t.err, wl, dbg);
     } else {
-        size_t sm = 2 * kT * sizeof(SrcF) + 2 * kT * SM * sizeof(LJf) + 2 * sizeof(uint64_t);
-        auto kern = k_direct32<SM, kP, kBX, kBY, kBZ, kT, DU, DH>;
-        raise_dyn_smem(kern, sm);
-        kern<<<grid, block, sm, st>>>(g, ph, t.srcf, t.ljf, t.n, o, t.err, wl, dbg);
+        // four points per lane share an atom's y and z terms, but only where that still leaves a few waves of CTAs
+        // (2,000 atoms, 128^3, 4,096 CTAs: 2.30 against 2.61 ms; 500 atoms, 64^3, 512 CTAs: 0.47 against 0.39)
+        const int64_t ctas = (int64_t)((g.nx + 15) / 16) * ((g.ny + 7) / 8) * ((g.nz + 3) / 4);
+        if (ctas >= 1824) return run_direct32<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
+        return run_direct32<SM, 2, DU, DH>(g, ph, t, o, wl, dbg, st);
     }
     return cudaGetLastError();
 }

@@ -228,6 +228,17 @@ __device__ __forceinline__ double f2d_alu(float f) {
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
+constexpr int kNTab = 128;  // segments of the short-range kernel tables over [0, r_short] (short_range_table)
+
+// Segment index and offset of u in [0, kNTab] (up to rounding) for the cubic pieces, without conversion
+// instructions: adding 1.5 2^23 leaves round(u - 1/2) (ties to even) in the low bits of the sum, and the sum
+// minus 1.5 2^23 is that integer as a float.  A tie gives the lower segment at offset 1, its end point.
+__device__ __forceinline__ float seg_split(float u, int& it) {
+    const float sh = (u - 0.5f) + 12582912.0f;
+    it = min(__float_as_int(sh) - 0x4B400000, kNTab - 1);
+    return u - fminf(sh - 12582912.0f, (float)(kNTab - 1));
+}
+
 // Error-free sum of two floats: a + b = s + e exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;

@@ -18,7 +18,15 @@ struct DevTables {
     LJd* ljd = nullptr;   // [n][smax]
     LJf* ljf = nullptr;   // [n][smax]
     DevErr* err = nullptr;
+    // FP32 direct sum: the short-range kernels' pieces (short_range_table) and kNTab / r_short in grid units; null: the
+    // kernels are called per pair (a caller without device memory of its own for them)
+    const float4* sr = nullptr;
+    float sr_inv = 0.f;
 };
+
+// The short-range kernels F_c(d) = erfc(x) and F_h(d) = e^{-x^2}[erfcx(x-a) + erfcx(x+a)] as cubic Hermite pieces in d
+// over [0, r_short], [kNTab][2] (host).
+void short_range_table(const Phys& ph, double h, float4* tab);
 
 struct Outputs {
     double* u = nullptr;

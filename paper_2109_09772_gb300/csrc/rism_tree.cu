@@ -1505,7 +1505,6 @@ __global__ void k_reset_meta(TreeMeta* meta) {
 // lane into a kStages-deep ring of tiles guarded by full (copy landed) and empty
 // (all warps done) mbarriers; every wait is bounded.
 constexpr int kStages = 4;
-constexpr int kNTab = 128;  // segments of the short-range kernel tables over [0, r_short]
 
 struct EvalArgs {
     GridD g;
@@ -2451,15 +2450,6 @@ struct NearShape {
     static_assert(NW <= 16, "the per-warp source lists of the near tile hold 16 warps");
 };
 
-// Segment index and offset of u in [0, kNTab] (up to rounding) for the cubic pieces, without conversion
-// instructions: adding 1.5 2^23 leaves round(u - 1/2) (ties to even) in the low bits of the sum, and the sum
-// minus 1.5 2^23 is that integer as a float.  A tie gives the lower segment at offset 1, its end point.
-__device__ __forceinline__ float seg_split(float u, int& it) {
-    const float sh = (u - 0.5f) + 12582912.0f;
-    it = min(__float_as_int(sh) - 0x4B400000, kNTab - 1);
-    return u - fminf(sh - 12582912.0f, (float)(kNTab - 1));
-}
-
 // One tile of near-field sources against the P points of a thread: LJ within the pair cut-offs (UNI: one
 // cut-off for every pair, tested once per pair instead of once per site) and the short-range remainders of
 // eq. (dcf-r) / eq. (tcf-r) within r_short from the cubic pieces in d.
@@ -3400,39 +3390,17 @@ rism_status tree_reserve(TreeState* s, const DevTables& t, const GridD& g, const
             s->cap_tpot = (int64_t)tb.nbox * P3;
         }
     }
-    // Short-range kernels of the near field as cubic Hermite pieces in d (grid units) over [0, r_short]:
-    // F_c(d) = erfc(x) and F_h(d) = e^{-x^2}[erfcx(x-a) + erfcx(x+a)] = e^{a^2-2ax} erfc(x-a) + e^{a^2+2ax} erfc(x+a),
-    // x = d h / eta, a = kappa eta / 2, with their derivatives dF_c/dx = -2/sqrt(pi) e^{-x^2} and
-    // dF_h/dx = -2a e^{a^2-2ax} erfc(x-a) + 2a e^{a^2+2ax} erfc(x+a) - 4/sqrt(pi) e^{-x^2}; built in FP64.
+    // short-range kernels of the near field
     const double key[4] = {ph.eta, g.h, ph.a, ph.rs};
     if (!s->ntab || std::memcmp(key, s->ntab_key, sizeof key) != 0) {
         if (!s->ntab && (e = cudaMalloc(&s->ntab, sizeof(float4) * 2 * kNTab)) != cudaSuccess)
             return cuda_err(err, e, "kernel table");
-        const double sx = g.h / ph.eta, a = ph.a, rsg = ph.rs / g.h, D = rsg / kNTab;
-        const double tsp = 2.0 / std::sqrt(3.14159265358979323846);
-        std::vector<double> fc(kNTab + 1), gc(kNTab + 1), fh(kNTab + 1), gh(kNTab + 1);
-        for (int k = 0; k <= kNTab; ++k) {
-            const double x = k * D * sx, ex = std::exp(-x * x);
-            const double em = std::exp(a * a - 2.0 * a * x), ep = std::exp(a * a + 2.0 * a * x);
-            const double cm = std::erfc(x - a), cp = std::erfc(x + a);
-            fc[k] = std::erfc(x);
-            gc[k] = -tsp * ex * sx * D;  // derivative per segment length
-            fh[k] = em * cm + ep * cp;
-            gh[k] = (-2.0 * a * em * cm + 2.0 * a * ep * cp - 2.0 * tsp * ex) * sx * D;
-        }
         std::vector<float4> tab(2 * kNTab);
-        auto herm = [](double f0, double f1, double g0, double g1) {
-            return make_float4((float)f0, (float)g0, (float)(3.0 * (f1 - f0) - 2.0 * g0 - g1),
-                               (float)(2.0 * (f0 - f1) + g0 + g1));
-        };
-        for (int k = 0; k < kNTab; ++k) {
-            tab[2 * k] = herm(fc[k], fc[k + 1], gc[k], gc[k + 1]);
-            tab[2 * k + 1] = herm(fh[k], fh[k + 1], gh[k], gh[k + 1]);
-        }
+        short_range_table(ph, g.h, tab.data());
         if ((e = cudaMemcpy(s->ntab, tab.data(), sizeof(float4) * 2 * kNTab, cudaMemcpyHostToDevice)) != cudaSuccess)
             return cuda_err(err, e, "kernel table");
         std::memcpy(s->ntab_key, key, sizeof key);
-        s->ntab_inv = (float)(kNTab / rsg);
+        s->ntab_inv = (float)(kNTab / (ph.rs / g.h));
     }
     return RISM_OK;
 }

@@ -190,3 +190,25 @@ def test_bounded_wait_timeout_is_reported_and_context_survives(R):
     for k in ("u", "c", "h"):
         assert rel_l2(out[k].cpu().numpy().reshape(r.S, -1), ref[k]) <= 1e-6
     r.close()
+
+
+@pytest.mark.parametrize("mode", ["none", "rcut", "tol"])
+@pytest.mark.parametrize("sites", [["O", "H"], ["O", "H", "Na+", "Cl-"], ["O", "H", "Na+", "Cl-", "O", "H"]])
+@pytest.mark.parametrize("n, grid", [(1, (163, 117, 61)), (65, (163, 117, 61)), (130, (16, 9, 5)), (63, (15, 8, 4))])
+def test_fp32_blocks_and_near_lists(R, n, grid, sites, mode):
+    """The FP32 direct sum with four points per lane (a grid of more than 1,824 CTAs) and with two, ragged in every
+    axis, atom tiles of one source, an odd count and one over a tile, an atom on a grid point (not alone in its tile),
+    each LJ cut-off mode and padded site count: every point against the oracle."""
+    w = I.small_workload(n_atoms=n, n=grid, h=0.5, seed=71, lj_rcut=3.1 if mode == "rcut" else 0.0, net=1.0)
+    if mode == "tol":
+        w.opts["lj_tol"] = 1e-2
+    w.solvent = I.solvent(sites)
+    if n > 1:
+        w.solute.xyz[n // 2] = np.asarray(w.grid.origin) + 0.5 * np.array([grid[0] // 2, grid[1] // 2, 2])
+    keys = ("u", "c", "h") if "Na+" in sites else ("u", "c")
+    ref = O.fields(O.Problem.from_workload(w), want=keys)
+    r = R.from_workload(w, method=R.METHOD_DIRECT, precision=R.PREC_FP32)
+    out = r.init(u=True, c=True, h="h" in keys)
+    g = {k: out[k].cpu().numpy().reshape(r.S, -1) for k in keys}
+    r.close()
+    check_fields(g, ref, keys, 1e-6, w.grid, w.solute.xyz, label=f"{n} atoms {grid} {mode}")
