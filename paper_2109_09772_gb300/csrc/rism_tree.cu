@@ -1694,7 +1694,7 @@ struct ItemSrc {
     const LJf* ljs;
 };
 
-// Ring driver of a persistent CTA that works through a sequence of items (target batches): the producer lane
+// Ring driver of a persistent CTA that works through a sequence of items (target batches): the producer warp
 // fills the ring with the tiles of item after item without a pause (every item takes at least one tile, the
 // last one flagged; an item without sources gets one empty tile), so the next item's sources load while the
 // consumer warps finish the previous one.  next(n, item, src) gives the CTA's n-th item (false: none left);
@@ -1709,48 +1709,81 @@ __device__ int run_stream(R& r, long long wlim, DevErr* err, FN&& next, FX&& ext
     const int tid = threadIdx.x, lane = tid & 31;
     volatile int* abort_flag = &r.abort;
     if (tid >= NWARPS * 32) {
-        if (tid == NWARPS * 32) {
-            Cursor c;
-            c.produced = 0;
-            for (int s = 0; s < kStages; ++s) c.last_phase[s] = -1;
-            bool ok = true;
-            for (int n = 0; ok; ++n) {
-                int item = -1;
-                ItemSrc is{nullptr, 0, 0, nullptr, nullptr};
-                const bool have = next(n, item, is);
-                c.e = have ? is.e : 0;
-                c.e_end = have ? is.e_end : 0;
-                c.off = 0;
-                c.left = INT_MAX;
-                for (bool more = true, first = true; more; first = false) {
-                    const int t = c.produced, slot = t % kStages;
-                    if (t >= kStages && !mbar_wait_bounded(&r.empty[slot], (uint32_t)((t / kStages - 1) & 1), wlim)) {
-                        ok = false;
-                        break;
+        // The producer warp: lane 0 takes the items and keeps the barriers; the lanes hold 32 list entries at a time and
+        // each issues the copies of its own range (a near tile is a dozen ranges, two copies each: issued by one lane
+        // they took longer than the consumers need for the tile).
+        Cursor c;
+        c.produced = 0;
+        for (int s = 0; s < kStages; ++s) c.last_phase[s] = -1;
+        bool ok = true;
+        for (int n = 0; ok; ++n) {
+            int item = -1;
+            ItemSrc is{nullptr, 0, 0, nullptr, nullptr};
+            bool have = false;
+            if (lane == 0) have = next(n, item, is);
+            have = __shfl_sync(0xffffffffu, (int)have, 0) != 0;
+            item = __shfl_sync(0xffffffffu, item, 0);
+            is.e_end = __shfl_sync(0xffffffffu, is.e_end, 0);
+            is.ent = reinterpret_cast<const int2*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(is.ent), 0));
+            is.src = reinterpret_cast<const SrcF*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(is.src), 0));
+            is.ljs = reinterpret_cast<const LJf*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(is.ljs), 0));
+            int base = have ? __shfl_sync(0xffffffffu, is.e, 0) : is.e_end;  // first entry after the window
+            int2 en = make_int2(0, 0);  // the lane's entry of the window
+            int end = 0, tot = 0, pos = 0;  // sources up to and with it, in the window, taken from the window
+            for (bool more = true, first = true; more; first = false) {
+                const int t = c.produced, slot = t % kStages;
+                if (t >= kStages) {
+                    if (lane == 0) ok = mbar_wait_bounded(&r.empty[slot], (uint32_t)((t / kStages - 1) & 1), wlim);
+                    ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                }
+                if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
+                if (!ok) break;
+                if (have && first && lane == 0) extra(n, item, &r.full[slot]);
+                int filled = 0;
+                while (filled < kT && (pos < tot || base < is.e_end)) {
+                    if (pos >= tot) {
+                        en = base + lane < is.e_end ? is.ent[base + lane] : make_int2(0, 0);
+                        base += 32;
+                        end = en.y;
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int v = __shfl_up_sync(0xffffffffu, end, o);
+                            if (lane >= o) end += v;
+                        }
+                        tot = __shfl_sync(0xffffffffu, end, 31);
+                        pos = 0;
                     }
-                    if (*abort_flag) {
-                        ok = false;
-                        break;
+                    const int take = min(kT - filled, tot - pos);
+                    if (lane == 0)
+                        mbar_expect_tx_only(&r.full[slot], (uint32_t)(take * (sizeof(SrcF) + (LJ ? SM * sizeof(LJf) : 0))));
+                    __syncwarp();
+                    const int lo = max(end - en.y, pos), cnt = min(end, pos + take) - lo;
+                    if (cnt > 0) {
+                        const int at = en.x + lo - (end - en.y), to = filled + lo - pos;
+                        bulk_g2s(r.src[slot] + to, is.src + at, cnt * sizeof(SrcF), &r.full[slot]);
+                        if (LJ)
+                            bulk_g2s(r.lj[LJ ? slot : 0] + to * SM, is.ljs + (int64_t)at * SM, cnt * SM * sizeof(LJf),
+                                     &r.full[slot]);
                     }
-                    if (have && first) extra(n, item, &r.full[slot]);
-                    const int cnt = have ? fill_ranges<SM, LJ>(c, is.ent, is.src, is.ljs, r.src[slot],
-                                                               r.lj[LJ ? slot : 0], &r.full[slot])
-                                         : 0;
-                    more = have && c.e < c.e_end;
-                    r.cnt[slot] = cnt;
+                    filled += take;
+                    pos += take;
+                }
+                more = have && (pos < tot || base < is.e_end);
+                c.last_phase[slot] = t / kStages;
+                c.produced = t + 1;
+                __syncwarp();
+                if (lane == 0) {
+                    r.cnt[slot] = filled;
                     r.item[slot] = have ? item : -1;
                     r.last[slot] = more ? 0 : 1;
-                    c.last_phase[slot] = t / kStages;
-                    c.produced = t + 1;
                     mbar_arrive(&r.full[slot]);
                 }
-                if (!have) break;
             }
-            if (!ok) {
-                *abort_flag = 1;
-                report_error(err, DEV_TIMEOUT, WHERE_TREE_EVAL);
-                drain(r, c, wlim);
-            }
+            if (!have) break;
+        }
+        if (!ok && lane == 0) {
+            *abort_flag = 1;
+            report_error(err, DEV_TIMEOUT, WHERE_TREE_EVAL);
+            drain(r, c, wlim);
         }
         return kRingProducer;
     }
