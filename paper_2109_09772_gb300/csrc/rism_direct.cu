@@ -173,13 +173,15 @@ void short_range_table(const Phys& ph, double h, float4* tab) {
         fh[k] = em * cm + ep * cp;
         gh[k] = (-2.0 * a * em * cm + 2.0 * a * ep * cp - 2.0 * tsp * ex) * sx * D;
     }
-    auto herm = [](double f0, double f1, double g0, double g1) {
-        return make_float4((float)f0, (float)g0, (float)(3.0 * (f1 - f0) - 2.0 * g0 - g1),
-                           (float)(2.0 * (f0 - f1) + g0 + g1));
-    };
     for (int k = 0; k < kNTab; ++k) {
-        tab[2 * k] = herm(fc[k], fc[k + 1], gc[k], gc[k + 1]);
-        tab[2 * k + 1] = herm(fh[k], fh[k + 1], gh[k], gh[k + 1]);
+        auto c2 = [&](const std::vector<double>& f, const std::vector<double>& g) {
+            return (float)(3.0 * (f[k + 1] - f[k]) - 2.0 * g[k] - g[k + 1]);
+        };
+        auto c3 = [&](const std::vector<double>& f, const std::vector<double>& g) {
+            return (float)(2.0 * (f[k] - f[k + 1]) + g[k] + g[k + 1]);
+        };
+        tab[2 * k] = make_float4((float)fc[k], (float)fh[k], (float)gc[k], (float)gh[k]);
+        tab[2 * k + 1] = make_float4(c2(fc, gc), c2(fh, gh), c3(fc, gc), c3(fh, gh));
     }
 }
 
@@ -565,16 +567,9 @@ __global__ void __launch_bounds__(128, SM > 4 ? 2 : (P > 2 ? 3 : 4))
                         if (d2[p] > 0.f) {
                             const float ri = rsqrt_approx(d2[p]), qr = g0.w * ri;
                             if (sr) {
-                                int it;
-                                const float tt = seg_split(d2[p] * ri * sr_inv, it);
-                                if (DC) {
-                                    const float4 c = tab[2 * it];
-                                    ff_add(sch[p], scl[p], qr * fmaf(fmaf(fmaf(c.w, tt, c.z), tt, c.y), tt, c.x));
-                                }
-                                if (DH) {
-                                    const float4 c = tab[2 * it + 1];
-                                    ff_add(shh[p], shl[p], qr * fmaf(fmaf(fmaf(c.w, tt, c.z), tt, c.y), tt, c.x));
-                                }
+                                const float2 f = up2(short_range(tab, d2[p] * ri * sr_inv));
+                                if (DC) ff_add(sch[p], scl[p], qr * f.x);
+                                if (DH) ff_add(shh[p], shl[p], qr * f.y);
                             } else {
                                 const float x = d2[p] * ri * xs;
                                 if (DC) ff_add(sch[p], scl[p], qr * erfcf(x));

@@ -203,6 +203,13 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float v) {
     lo += t;
 }
 
+// The same on two independent sums, one per half.
+__device__ __forceinline__ void ff_add2(f32x2& hi, f32x2& lo, f32x2 v) {
+    const f32x2 s = add2(hi, v), bb = sub2(s, hi);
+    lo = add2(lo, add2(sub2(hi, sub2(s, bb)), sub2(v, bb)));
+    hi = s;
+}
+
 // float -> double on the integer pipe (the FP64 pipe of this part is slow).  Normal numbers: sign, exponent
 // rebiased by 1023 - 127 = 896, fraction shifted left by 52 - 23 = 29.  The rare rest, out of line so that the
 // common path stays short: all-ones exponent (infinity, NaN) kept all-ones, zero kept zero, a subnormal
@@ -228,7 +235,9 @@ __device__ __forceinline__ double f2d_alu(float f) {
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
-constexpr int kNTab = 128;  // segments of the short-range kernel tables over [0, r_short] (short_range_table)
+// Short-range kernel tables over [0, r_short] (short_range_table): segment k holds the coefficients of both kernels as
+// two-wide operands, (c0, h0, c1, h1) and (c2, h2, c3, h3).
+constexpr int kNTab = 128;
 
 // Segment index and offset of u in [0, kNTab] (up to rounding) for the cubic pieces, without conversion
 // instructions: adding 1.5 2^23 leaves round(u - 1/2) (ties to even) in the low bits of the sum, and the sum
@@ -237,6 +246,16 @@ __device__ __forceinline__ float seg_split(float u, int& it) {
     const float sh = (u - 0.5f) + 12582912.0f;
     it = min(__float_as_int(sh) - 0x4B400000, kNTab - 1);
     return u - fminf(sh - 12582912.0f, (float)(kNTab - 1));
+}
+
+// (F_c, F_h) at u = d kNTab / r_short.
+__device__ __forceinline__ f32x2 short_range(const float4* tab, float u) {
+    int it;
+    const float tt = seg_split(u, it);
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&tab[2 * it]);
+    const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&tab[2 * it + 1]);
+    const f32x2 T = pk2(tt, tt);
+    return fma2(fma2(fma2(b.y, T, b.x), T, a.y), T, a.x);
 }
 
 // Error-free sum of two floats: a + b = s + e exactly.
