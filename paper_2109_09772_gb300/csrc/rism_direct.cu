@@ -188,9 +188,9 @@ void short_range_table(const Phys& ph, double h, float4* tab) {
 // ------------------------------------------------------- common epilogue
 template <int P>
 __device__ __forceinline__ void store_strip(double* base, int i0, int nx, const double (&v)[P], bool vec_ok) {
-    if (vec_ok && i0 + P <= nx) {
+    if (P % 2 == 0 && vec_ok && i0 + P <= nx) {
 #pragma unroll
-        for (int p = 0; p < P; p += 2)
+        for (int p = 0; p + 1 < P; p += 2)
             __stcs(reinterpret_cast<double2*>(base + i0 + p), make_double2(v[p], v[p + 1]));
     } else {
 #pragma unroll
@@ -199,21 +199,42 @@ __device__ __forceinline__ void store_strip(double* base, int i0, int nx, const 
     }
 }
 
+constexpr int kDirectT = 64;  // atoms per tile (two ballots)
+
 // ------------------------------------------------------------ FP64 direct
-// Launch shape: BX x BY x BZ threads, P x-points per thread, T atoms per tile.
-template <int SM, int P, int BX, int BY, int BZ, int T, bool DU, bool DH>
-__global__ void __launch_bounds__(BX* BY* BZ) k_direct64(GridD g, Phys ph, const Geo* __restrict__ geo,
-                                                          const LJd* __restrict__ lj, int64_t n, Outputs o,
-                                                          DevErr* err, long long wlim, int dbg) {
-    constexpr int NT = BX * BY * BZ;
+// The FP64 pipe of this part is slow (1.7 multiply-adds per clock per SM), so what need not run on it does not:
+// comparisons of non-negative doubles order their bit patterns on the integer pipe.
+__device__ __forceinline__ bool lt_bits(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+
+// 1/sqrt(d2) (0 for d2 = 0): the single-precision approximation of the leading bits, moved to and from FP32 by their bit
+// patterns, and one step of Halley's iteration: with h = 1 - d2 y^2, y + y h (1/2 + 3/8 h) leaves 5/16 h^3, below 2^-64;
+// five FP64 operations.  Exponents outside FP32's range take the library function.
+__device__ __noinline__ double rsqrt64_slow(double d2) { return d2 > 0.0 ? rsqrt(d2) : 0.0; }
+__device__ __forceinline__ double rsqrt64(double d2) {
+    const uint32_t hi = (uint32_t)__double2hiint(d2), lo = (uint32_t)__double2loint(d2);
+    if ((hi >> 20) - 910u > 220u) return rsqrt64_slow(d2);
+    const uint32_t f = __float_as_uint(rsqrt_approx(__uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29))));
+    const double y = __hiloint2double((int)((f >> 3) + 0x38000000u), (int)(f << 29));
+    const double h = fma(-(d2 * y), y, 1.0);
+    return fma(y * h, fma(h, 0.375, 0.5), y);
+}
+
+// Launch shape: four warps of 8 x 4 x 4 points (P = 4) or 2 x 4 x 4 (P = 1), two by two along x and y; T atoms per tile.
+// A warp's points are compact so that few warps take an atom's erfc remainders for the sake of a few of their points.
+// Bound by the FP64 pipe.  200 atoms on 64^3, two sites, no cut-off: DIRECT64 ms (4.2 ms with the library's reciprocal
+// square root, a division per pair, comparisons in FP64 and warps of 32 x 4 x 1 points).
+template <int SM, int P, int T, bool DU, bool DH>
+__global__ void __launch_bounds__(128) k_direct64(GridD g, Phys ph, const Geo* __restrict__ geo,
+                                                  const LJd* __restrict__ lj, int64_t n, Outputs o, DevErr* err,
+                                                  long long wlim, int dbg) {
     extern __shared__ __align__(16) unsigned char smem[];
     Geo* sgeo = reinterpret_cast<Geo*>(smem);
     LJd* slj = reinterpret_cast<LJd*>(smem + 2 * T * sizeof(Geo));
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * T * sizeof(Geo) + 2 * T * SM * sizeof(LJd));
 
-    const int tid = threadIdx.x;
-    const int tx = tid % BX, ty = (tid / BX) % BY, tz = tid / (BX * BY);
-    const int i0 = (blockIdx.x * BX + tx) * P, j = blockIdx.y * BY + ty, k = blockIdx.z * BZ + tz;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int i0 = (blockIdx.x * 2 + (w & 1)) * 2 * P + (lane & 1) * P;
+    const int j = (blockIdx.y * 2 + (w >> 1)) * 4 + ((lane >> 1) & 3), k = blockIdx.z * 4 + (lane >> 3);
     double gx[P];
 #pragma unroll
     for (int p = 0; p < P; ++p) gx[p] = g.ox + g.h * (double)(i0 + p);
@@ -272,12 +293,12 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct64(GridD g, Phys ph, const
             for (int p = 0; p < P; ++p) {
                 const double dx = gx[p] - A.x;
                 const double d2 = fma(dx, dx, dyz2);
-                const double ri = d2 > 0.0 ? rsqrt(d2) : 0.0;
+                const double ri = rsqrt64(d2);
                 const double qr = A.q * ri;
                 f1[p] += qr;
                 if (DH) fk[p] += qr * exp(-kap * (d2 * ri));
-                if (d2 < rs2) {
-                    if (d2 > 0.0) {
+                if (lt_bits(d2, rs2)) {
+                    if (__double_as_longlong(d2) != 0ll) {
                         const double x = d2 * ri * ieta;
                         if (DC) sc[p] += qr * erfc(x);
                         if (DH) sh[p] += qr * exp(-x * x) * (erfcx(x - a) + erfcx(x + a));
@@ -288,12 +309,18 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct64(GridD g, Phys ph, const
                     }
                 }
                 if (DU) {
-                    const double r2i = 1.0 / d2;
-                    const double r6 = r2i * r2i * r2i;
+                    long long rc = 0ll;  // the largest cut-off of the atom's sites
 #pragma unroll
-                    for (int s = 0; s < SM; ++s) {
-                        const LJd l = L[aa * SM + s];
-                        if (d2 < l.rc2) lj_[p][s] += r6 * (l.A * r6 - l.B);
+                    for (int s = 0; s < SM; ++s) rc = max(rc, __double_as_longlong(L[aa * SM + s].rc2));
+                    if (__double_as_longlong(d2) < rc) {
+                        // 1/d^2 from the square of the reciprocal root with the residual made up: three operations
+                        const double y2 = ri * ri, r2i = fma(y2, fma(-d2, y2, 1.0), y2);
+                        const double r6 = r2i * r2i * r2i;
+#pragma unroll
+                        for (int s = 0; s < SM; ++s) {
+                            const LJd l = L[aa * SM + s];
+                            if (lt_bits(d2, l.rc2)) lj_[p][s] += r6 * (l.A * r6 - l.B);
+                        }
                     }
                 }
             }
@@ -304,7 +331,7 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct64(GridD g, Phys ph, const
     if (j >= g.ny || k >= g.nz || i0 >= g.nx) return;
     const int64_t plane = (int64_t)g.nx * g.ny * g.nz;
     const int64_t row = ((int64_t)k * g.ny + j) * g.nx;
-    const bool vec_ok = (g.nx & 1) == 0;
+    const bool vec_ok = P > 1 && (g.nx & 1) == 0;
     const double cu0 = ph.k_e, cc0 = -ph.beta * ph.k_e, ch0 = -ph.beta * ph.k_e / (2.0 * ph.eps_r);
 #pragma unroll
     for (int s = 0; s < SM; ++s) {
@@ -339,7 +366,6 @@ __global__ void __launch_bounds__(BX* BY* BZ) k_direct64(GridD g, Phys ph, const
 // atoms a warp takes the long-range sums of all of them, two sources per instruction, and then only the atoms within
 // the short-range radius or their largest LJ cut-off of its block, listed by ballots, for the LJ terms and the erfc
 // remainders (a few in a hundred of a solute's atoms).
-constexpr int kDirectT = 64;  // atoms per tile (two ballots)
 
 // Sources 2l and 2l + 1 of a tile, field by field (two-wide operands); an odd count is padded with a zero charge 10^6
 // grid units away, whose terms are exactly zero.
@@ -636,8 +662,6 @@ __global__ void __launch_bounds__(128, SM > 4 ? 2 : (P > 2 ? 3 : 4))
 
 // ---------------------------------------------------------------- launch
 namespace {
-constexpr int kP = 4, kBX = 8, kBY = 4, kBZ = 4, kT = 64;
-
 template <int SM, int P, bool DU, bool DH>
 cudaError_t run_direct32(const GridD& g, const Phys& ph, const DevTables& t, Outputs o, long long wl, int dbg,
                          cudaStream_t st) {
@@ -649,24 +673,30 @@ cudaError_t run_direct32(const GridD& g, const Phys& ph, const DevTables& t, Out
     return cudaGetLastError();
 }
 
+template <int SM, int P, bool DU, bool DH>
+cudaError_t run_direct64(const GridD& g, const Phys& ph, const DevTables& t, Outputs o, long long wl, int dbg,
+                         cudaStream_t st) {
+    const size_t sm = 2 * kDirectT * sizeof(Geo) + 2 * kDirectT * SM * sizeof(LJd) + 2 * sizeof(uint64_t);
+    const dim3 grid((g.nx + 4 * P - 1) / (4 * P), (g.ny + 7) / 8, (g.nz + 3) / 4);
+    auto kern = k_direct64<SM, P, kDirectT, DU, DH>;
+    raise_dyn_smem(kern, sm);
+    kern<<<grid, 128, sm, st>>>(g, ph, t.geo, t.ljd, t.n, o, t.err, wl, dbg);
+    return cudaGetLastError();
+}
+
 template <int SM, bool DU, bool DH>
 cudaError_t run_direct(const GridD& g, const Phys& ph, const DevTables& t, int prec, Outputs o, long long wl,
                        int dbg, cudaStream_t st) {
-    dim3 grid((g.nx + kBX * kP - 1) / (kBX * kP), (g.ny + kBY - 1) / kBY, (g.nz + kBZ - 1) / kBZ);
-    dim3 block(kBX * kBY * kBZ);
+    const int64_t ctas = (int64_t)((g.nx + 15) / 16) * ((g.ny + 7) / 8) * ((g.nz + 3) / 4);  // four points per lane
     if (prec == RISM_PREC_FP64) {
-        size_t sm = 2 * kT * sizeof(Geo) + 2 * kT * SM * sizeof(LJd) + 2 * sizeof(uint64_t);
-        auto kern = k_direct64<SM, kP, kBX, kBY, kBZ, kT, DU, DH>;
-        raise_dyn_smem(kern, sm);
-        kern<<<grid, block, sm, st>>>(g, ph, t.geo, t.ljd, t.n, o, t.err, wl, dbg);
-    } else {
-        // four points per lane share an atom's y and z terms, but only where that still leaves a few waves of CTAs
-        // (2,000 atoms, 128^3, 4,096 CTAs: 2.30 against 2.61 ms; 500 atoms, 64^3, 512 CTAs: 0.47 against 0.39)
-        const int64_t ctas = (int64_t)((g.nx + 15) / 16) * ((g.ny + 7) / 8) * ((g.nz + 3) / 4);
-        if (ctas >= 1824) return run_direct32<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
-        return run_direct32<SM, 2, DU, DH>(g, ph, t, o, wl, dbg, st);
+        // one point per lane where four would leave SMs without work (FP64 pipes idle)
+        if (ctas >= 2 * 152) return run_direct64<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
+        return run_direct64<SM, 1, DU, DH>(g, ph, t, o, wl, dbg, st);
     }
-    return cudaGetLastError();
+    // four points per lane share an atom's y and z terms, but only where that still leaves a few waves of CTAs (2,000
+    // atoms, 128^3, 4,096 CTAs: 2.30 against 2.61 ms; 500 atoms, 64^3, 512 CTAs: 0.47 against 0.39)
+    if (ctas >= 1824) return run_direct32<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
+    return run_direct32<SM, 2, DU, DH>(g, ph, t, o, wl, dbg, st);
 }
 
 template <int SM>

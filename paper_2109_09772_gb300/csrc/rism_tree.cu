@@ -4789,18 +4789,27 @@ __global__ void __launch_bounds__(256) k_adj_qagg(TBoxes tb, int l, const float2
     const int sp = 1 << l;
     const int r0x = ib * sp, r0y = jb * sp, r0z = kb * sp;
     const int r1x = min(r0x + sp, tb.nbx[0]), r1y = min(r0y + sp, tb.nby[0]), r1z = min(r0z + sp, tb.nbz[0]);
-    for (int rz = r0z; rz < r1z; ++rz)
-        for (int ry = r0y; ry < r1y; ++ry)
-            for (int rx = r0x; rx < r1x; ++rx) {
-                const int rb = (rz * tb.nby[0] + ry) * tb.nbx[0] + rx;
-                if (rlow[rb] != l) continue;
-                const float2* src = qpart + (int64_t)rb * P3;
-                for (int k = threadIdx.x; k < P3; k += blockDim.x) {
-                    const float2 v = src[k];
-                    acc[k].x += v.x;
-                    acc[k].y += v.y;
-                }
+    // The regions whose lowest box this is: above level 0 only a few at the grid's edges, so the threads look through
+    // them side by side (one after the other, the 9,600 regions of a root box took half a millisecond).
+    __shared__ int found[256];
+    const int nrx = r1x - r0x, nry = r1y - r0y, nr = nrx * nry * (r1z - r0z);
+    for (int b0 = 0; b0 < nr; b0 += blockDim.x) {
+        const int i = b0 + threadIdx.x;
+        const int rb = ((r0z + i / (nrx * nry)) * tb.nby[0] + r0y + (i / nrx) % nry) * tb.nbx[0] + r0x + i % nrx;
+        const bool mine = i < nr && rlow[rb] == l;
+        found[threadIdx.x] = mine ? rb : -1;
+        if (!__syncthreads_or(mine)) continue;
+        for (int j = 0; j < min((int)blockDim.x, nr - b0); ++j) {  // in region order
+            if (found[j] < 0) continue;
+            const float2* src = qpart + (int64_t)found[j] * P3;
+            for (int k = threadIdx.x; k < P3; k += blockDim.x) {
+                const float2 v = src[k];
+                acc[k].x += v.x;
+                acc[k].y += v.y;
             }
+        }
+        __syncthreads();
+    }
     __syncthreads();
     if (l > 0) {
         for (int c = 0; c < 8; ++c) {

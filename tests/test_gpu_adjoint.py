@@ -333,3 +333,25 @@ def test_near_columns_vs_oracle(R, mode, n, sites):
         b = _gpu_grad(R, w, G)
         for k in ("sigma", "eps"):
             assert np.array_equal(b[k][far], g[k][far]) and np.isnan(b[k][d < 3.5]).all()
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-12, 1e10])
+def test_cotangent_scales_and_wide_boxes(R, scale):
+    """Cotangents far from 1 (their FP32 split ends at 2^-93, smaller ones take the FP64 pipe) with exact zeros among
+    them: the gradients scale with them.  The grid has boxes above level 0 that hold clipped regions of their own."""
+    import torch
+
+    w = I.small_workload(n_atoms=120, n=(70, 37, 35), h=0.5, seed=81, ions=True, lj_rcut=5.0, net=1.0)
+    G = _cotangents(w, 29)
+    for k in G:
+        G[k][:, ::5] = 0.0
+    def run(f):
+        r = R.from_workload(w, method=R.METHOD_TREECODE, precision=R.PREC_FP32)
+        g = r.backward(*(torch.as_tensor(f * G[k], device="cuda") for k in ("u", "c", "h")))
+        r.close()
+        return {k: v.cpu().numpy() for k, v in g.items()}
+    one, got = run(1.0), run(scale)
+    ref = O.grad(O.Problem.from_workload(w), np.arange(120), G["u"], G["c"], G["h"])
+    _check(one, ref, np.arange(120))
+    for k in one:
+        assert rel_l2(got[k] / scale, one[k]) <= GRAD_TOL
