@@ -649,7 +649,7 @@ static cudaError_t near_table(AdjointState* s, const GridD& g, const Phys& ph) {
     return cudaSuccess;
 }
 
-rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, const GridD& g, const Phys& ph,
+rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, const GridD& g, const Phys& ph_,
                         const rism_options& o, const double* raw_dev, const double* sig_s, const double* eps_s,
                         const double* g_u, const double* g_c, const double* g_h, double* d_xyz, double* d_q,
                         double* d_sigma, double* d_eps, cudaStream_t st, std::string& err) {
@@ -657,6 +657,9 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
         err = "the adjoint is implemented with FP32 pair terms (precision RISM_PREC_FP32)";
         return RISM_E_UNSUPPORTED;
     }
+    // the short-range kernels end at (5 + a) eta for FP32 (2e-12 of the whole): a wider r_short does not stretch the pieces
+    Phys ph = ph_;
+    ph.rs = std::min(ph.rs, (5.0 + ph.a) * ph.eta);
     const int n = (int)t.n;
     if (n == 0) return RISM_OK;
     const int64_t M = (int64_t)g.nx * g.ny * g.nz;

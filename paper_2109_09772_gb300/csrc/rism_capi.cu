@@ -46,7 +46,7 @@ struct rism_ctx {
     DevErr* d_err = nullptr;
     DevErr* h_err = nullptr;  // pinned
     double* d_tail = nullptr;
-    float4* d_sr = nullptr;  // short-range pieces of the FP32 direct sum, built for sr_key
+    void* d_sr = nullptr;  // short-range pieces of the direct sum, built for sr_key
     double sr_key[4] = {0.0, 0.0, 0.0, -1.0};
     // the solute, [n][6] x, y, z, q, sigma, eps, in page-locked host memory: uploaded as it stands (by the
     // replayed graph's copy node or an asynchronous copy); every entry point that uploads it synchronises its
@@ -170,19 +170,29 @@ rism_status reserve_tables(rism_ctx* c) {
     c->t.err = c->d_err;
     c->gd = GridD{c->g.nx, c->g.ny, c->g.nz, c->g.h, c->g.origin[0], c->g.origin[1], c->g.origin[2]};
     make_phys(c);
-    if (c->o.method == RISM_METHOD_DIRECT && c->o.precision == RISM_PREC_FP32) {
-        const double key[4] = {c->ph.eta, c->gd.h, c->ph.a, c->ph.rs};
+    c->t.sr = nullptr;
+    c->t.sr64 = nullptr;
+    if (c->o.method == RISM_METHOD_DIRECT && short_pieces(c->ph)) {  // the short-range pieces, of the options' precision
+        const bool f64 = c->o.precision == RISM_PREC_FP64;
+        Phys ph = c->ph;
+        ph.rs = short_reach(ph, f64);
+        const double key[4] = {ph.eta, c->gd.h, ph.a, ph.rs};
+        const size_t bytes = f64 ? sizeof(double) * kLen64 : sizeof(float4) * 2 * kNTab;
         if (!c->d_sr || std::memcmp(key, c->sr_key, sizeof key) != 0) {
-            if (!c->d_sr && (e = cudaMalloc(&c->d_sr, sizeof(float4) * 2 * kNTab)) != cudaSuccess)
-                return cuda_fail(c, e, "short-range table");
-            std::vector<float4> tab(2 * kNTab);
-            short_range_table(c->ph, c->gd.h, tab.data());
-            if ((e = cudaMemcpy(c->d_sr, tab.data(), sizeof(float4) * tab.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+            if (!c->d_sr && (e = cudaMalloc(&c->d_sr, bytes)) != cudaSuccess) return cuda_fail(c, e, "short-range table");
+            std::vector<double> tab(bytes / sizeof(double));
+            if (f64) short_range_table64(ph, tab.data());
+            else short_range_table(ph, c->gd.h, reinterpret_cast<float4*>(tab.data()));
+            if ((e = cudaMemcpy(c->d_sr, tab.data(), bytes, cudaMemcpyHostToDevice)) != cudaSuccess)
                 return cuda_fail(c, e, "short-range table");
             std::memcpy(c->sr_key, key, sizeof key);
         }
-        c->t.sr = c->d_sr;
-        c->t.sr_inv = (float)(kNTab / (c->ph.rs / c->gd.h));
+        if (f64) {
+            c->t.sr64 = static_cast<const double*>(c->d_sr);
+        } else {
+            c->t.sr = static_cast<const float4*>(c->d_sr);
+            c->t.sr_inv = (float)(kNTab / (ph.rs / c->gd.h));
+        }
     }
     return RISM_OK;
 }

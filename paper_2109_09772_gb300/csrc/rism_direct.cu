@@ -185,6 +185,40 @@ void short_range_table(const Phys& ph, double h, float4* tab) {
     }
 }
 
+// Taylor pieces: in t = (u - middle) with u = d kTab64 / r_short, |t| <= 1/2.  With E = e^{-x^2} and H_k the Hermite
+// polynomials, E^(k) = (-1)^k H_k E; F_c' = -(2/sqrt(pi)) E; and F_h = G- + G+ with G-+ = e^{a^2 -+ 2ax} erfc(x -+ a),
+// G-+' = -+ 2a G-+ - (2/sqrt(pi)) E, differentiated term by term.  Eight terms leave less than 1e-16 (the segments are
+// 0.0234 eta wide at r_short = 6 eta).
+void short_range_table64(const Phys& ph, double* tab) {
+    const double a = ph.a, dx = ph.rs / ph.eta / kTab64, tsp = 2.0 / std::sqrt(3.14159265358979323846);
+    for (int s = 0; s < kTab64; ++s) {
+        const double x = (s + 0.5) * dx;
+        double E[kTerm64], hm = 0.0, h = 1.0;  // E^(k)
+        for (int k = 0; k < kTerm64; ++k) {
+            E[k] = (k & 1 ? -h : h) * std::exp(-x * x);
+            const double nx = 2.0 * x * h - 2.0 * k * hm;
+            hm = h;
+            h = nx;
+        }
+        double gm = std::exp(a * a - 2.0 * a * x) * std::erfc(x - a), gp = std::exp(a * a + 2.0 * a * x) * std::erfc(x + a);
+        double c = std::erfc(x), f = 1.0;  // f = dx^k / k!
+        for (int k = 0; k < kTerm64; ++k) {
+            tab[s * kTerm64 + k] = c * f;
+            tab[(kTab64 + s) * kTerm64 + k] = (gm + gp) * f;
+            c = -tsp * E[k];
+            gm = -2.0 * a * gm - tsp * E[k];
+            gp = 2.0 * a * gp - tsp * E[k];
+            f *= dx / (k + 1);
+        }
+    }
+    for (int j = 0; j < 256; ++j) {  // 2^(j/256) as a double and what its rounding left (long double's extra digits)
+        const long double v = std::exp2((long double)j / 256.0L);
+        double* o = tab + 2 * kTab64 * kTerm64 + 2 * j;
+        o[0] = (double)v;
+        o[1] = (double)(v - (long double)o[0]);
+    }
+}
+
 // ------------------------------------------------------- common epilogue
 template <int P>
 __device__ __forceinline__ void store_strip(double* base, int i0, int nx, const double (&v)[P], bool vec_ok) {
@@ -219,20 +253,51 @@ __device__ __forceinline__ double rsqrt64(double d2) {
     return fma(y * h, fma(h, 0.375, 0.5), y);
 }
 
+constexpr double kRound64 = 6755399441055744.0;  // 1.5 2^52: adding it leaves round(v) in the low word
+
+// F at u = d kTab64 / r_short (below kTab64) from a table of short_range_table64.
+__device__ __forceinline__ double piece64(const double* tab, double u) {
+    const double m = (u - 0.5) + kRound64;  // the segment: round(u - 1/2)
+    const int it = min(__double2loint(m), kTab64 - 1);
+    const double t = (u - 0.5) - (it == __double2loint(m) ? m - kRound64 : (double)(kTab64 - 1));
+    const double2* c = reinterpret_cast<const double2*>(tab + it * kTerm64);
+    const double2 c67 = c[3], c45 = c[2], c23 = c[1], c01 = c[0];
+    return fma(fma(fma(fma(fma(fma(fma(c67.y, t, c67.x), t, c45.y), t, c45.x), t, c23.y), t, c23.x), t, c01.y), t, c01.x);
+}
+
+// e^{-kappa d} from c = -256 kappa log2(e): with N = round(c d) and f = c d - N, 2^(N/256) as a pair from the table and
+// the powers of two, e^{f ln2/256} from four terms (below 4e-17); ten FP64 operations with the distance.
+__device__ __forceinline__ double exp64(const double2* pow2, double d, double c) {
+    const double m = fma(d, c, kRound64);
+    const int n = __double2loint(m);
+    const double f = fma(d, c, -(m - kRound64));
+    constexpr double L = 0.69314718055994530942 / 256.0;
+    const double p = fma(fma(fma(L * L * L * L / 24.0, f, L * L * L / 6.0), f, L * L / 2.0), f, L);
+    const double2 t = pow2[n & 255];
+    const double e = t.x + fma(t.x, f * p, t.y);
+    return n < -261000 || d * c < -1e9 ? 0.0 : __hiloint2double(__double2hiint(e) + (n >> 8) * (1 << 20), __double2loint(e));
+}
+
 // Launch shape: four warps of 8 x 4 x 4 points (P = 4) or 2 x 4 x 4 (P = 1), two by two along x and y; T atoms per tile.
 // A warp's points are compact so that few warps take an atom's erfc remainders for the sake of a few of their points.
-// Bound by the FP64 pipe.  200 atoms on 64^3, two sites, no cut-off: DIRECT64 ms (4.2 ms with the library's reciprocal
-// square root, a division per pair, comparisons in FP64 and warps of 32 x 4 x 1 points).
+// Bound by the FP64 pipe.  200 atoms on 64^3, two sites, no cut-off: 2.4 ms (4.2 ms with the library's reciprocal
+// square root and erfc, a division per pair, comparisons in FP64 and warps of 32 x 4 x 1 points).
 template <int SM, int P, int T, bool DU, bool DH>
 __global__ void __launch_bounds__(128) k_direct64(GridD g, Phys ph, const Geo* __restrict__ geo,
-                                                  const LJd* __restrict__ lj, int64_t n, Outputs o, DevErr* err,
+                                                  const LJd* __restrict__ lj, int64_t n,
+                                                  const double* __restrict__ sr, Outputs o, DevErr* err,
                                                   long long wlim, int dbg) {
     extern __shared__ __align__(16) unsigned char smem[];
     Geo* sgeo = reinterpret_cast<Geo*>(smem);
     LJd* slj = reinterpret_cast<LJd*>(smem + 2 * T * sizeof(Geo));
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * T * sizeof(Geo) + 2 * T * SM * sizeof(LJd));
+    double* tab = reinterpret_cast<double*>(bar + 2);  // [kLen64]
+    const double2* pow2 = reinterpret_cast<const double2*>(tab + 2 * kTab64 * kTerm64);
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    if (sr)
+        for (int q = tid; q < kLen64; q += 128) tab[q] = sr[q];
+    const double srinv = kTab64 / ph.rs, kexp = -256.0 * 1.4426950408889634074 * ph.kappa;
     const int i0 = (blockIdx.x * 2 + (w & 1)) * 2 * P + (lane & 1) * P;
     const int j = (blockIdx.y * 2 + (w >> 1)) * 4 + ((lane >> 1) & 3), k = blockIdx.z * 4 + (lane >> 3);
     double gx[P];
@@ -296,10 +361,14 @@ __global__ void __launch_bounds__(128) k_direct64(GridD g, Phys ph, const Geo* _
                 const double ri = rsqrt64(d2);
                 const double qr = A.q * ri;
                 f1[p] += qr;
-                if (DH) fk[p] += qr * exp(-kap * (d2 * ri));
+                const double d = d2 * ri;
+                if (DH) fk[p] += qr * (sr ? exp64(pow2, d, kexp) : exp(-kap * d));
                 if (lt_bits(d2, rs2)) {
-                    if (__double_as_longlong(d2) != 0ll) {
-                        const double x = d2 * ri * ieta;
+                    if (__double_as_longlong(d2) != 0ll && sr) {
+                        if (DC) sc[p] += qr * piece64(tab, d * srinv);
+                        if (DH) sh[p] += qr * piece64(tab + kTab64 * kTerm64, d * srinv);
+                    } else if (__double_as_longlong(d2) != 0ll) {
+                        const double x = d * ieta;
                         if (DC) sc[p] += qr * erfc(x);
                         if (DH) sh[p] += qr * exp(-x * x) * (erfcx(x - a) + erfcx(x + a));
                     } else {
@@ -676,11 +745,12 @@ cudaError_t run_direct32(const GridD& g, const Phys& ph, const DevTables& t, Out
 template <int SM, int P, bool DU, bool DH>
 cudaError_t run_direct64(const GridD& g, const Phys& ph, const DevTables& t, Outputs o, long long wl, int dbg,
                          cudaStream_t st) {
-    const size_t sm = 2 * kDirectT * sizeof(Geo) + 2 * kDirectT * SM * sizeof(LJd) + 2 * sizeof(uint64_t);
+    const size_t sm = 2 * kDirectT * sizeof(Geo) + 2 * kDirectT * SM * sizeof(LJd) + 2 * sizeof(uint64_t) +
+                      kLen64 * sizeof(double);
     const dim3 grid((g.nx + 4 * P - 1) / (4 * P), (g.ny + 7) / 8, (g.nz + 3) / 4);
     auto kern = k_direct64<SM, P, kDirectT, DU, DH>;
     raise_dyn_smem(kern, sm);
-    kern<<<grid, 128, sm, st>>>(g, ph, t.geo, t.ljd, t.n, o, t.err, wl, dbg);
+    kern<<<grid, 128, sm, st>>>(g, ph, t.geo, t.ljd, t.n, t.sr64, o, t.err, wl, dbg);
     return cudaGetLastError();
 }
 
@@ -689,8 +759,9 @@ cudaError_t run_direct(const GridD& g, const Phys& ph, const DevTables& t, int p
                        int dbg, cudaStream_t st) {
     const int64_t ctas = (int64_t)((g.nx + 15) / 16) * ((g.ny + 7) / 8) * ((g.nz + 3) / 4);  // four points per lane
     if (prec == RISM_PREC_FP64) {
-        // one point per lane where four would leave SMs without work (FP64 pipes idle)
-        if (ctas >= 2 * 152) return run_direct64<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
+        // one point per lane where four would be fewer than three waves of CTAs (200 atoms, two sites, one against four
+        // points: 32^3, 64 CTAs, 0.45 / 0.90 ms; 56^3, 392 CTAs, 1.79 / 1.94; 64^3, 512 CTAs, 2.46 / 2.41; 80^3 4.39 / 4.08)
+        if (ctas >= 3 * 152) return run_direct64<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
         return run_direct64<SM, 1, DU, DH>(g, ph, t, o, wl, dbg, st);
     }
     // four points per lane share an atom's y and z terms, but only where that still leaves a few waves of CTAs (2,000
@@ -712,9 +783,11 @@ cudaError_t run_direct_sm(const GridD& g, const Phys& ph, const DevTables& t, in
 
 int direct_variant_count() { return 1; }
 
-cudaError_t launch_direct(const GridD& g, const Phys& ph, const DevTables& t, int precision, Outputs o,
+cudaError_t launch_direct(const GridD& g, const Phys& ph_, const DevTables& t, int precision, Outputs o,
                           long long wait_limit, int variant, int dbg, cudaStream_t st) {
     (void)variant;
+    Phys ph = ph_;
+    if (t.sr || t.sr64) ph.rs = short_reach(ph, precision == RISM_PREC_FP64);
     switch (t.smax) {
         case 2: return run_direct_sm<2>(g, ph, t, precision, o, wait_limit, dbg, st);
         case 4: return run_direct_sm<4>(g, ph, t, precision, o, wait_limit, dbg, st);

@@ -22,11 +22,21 @@ struct DevTables {
     // kernels are called per pair (a caller without device memory of its own for them)
     const float4* sr = nullptr;
     float sr_inv = 0.f;
+    const double* sr64 = nullptr;  // the FP64 direct sum's (short_range_table64), null likewise
 };
 
 // The short-range kernels F_c(d) = erfc(x) and F_h(d) = e^{-x^2}[erfcx(x-a) + erfcx(x+a)] as cubic Hermite pieces in d
 // over [0, r_short], [kNTab][2] (host).
 void short_range_table(const Phys& ph, double h, float4* tab);
+// The same two kernels for FP64: kTab64 pieces of kTerm64 coefficients each (F_c then F_h) about the middle of their
+// segment of [0, r_short], then 2^(j/256) as pairs (host, kLen64 doubles).
+constexpr int kTab64 = 256, kTerm64 = 8, kLen64 = 2 * kTab64 * kTerm64 + 512;
+void short_range_table64(const Phys& ph, double* tab);
+// The pieces serve the direct sum for a = kappa eta/2 up to 1/2 (e^{-2ax} varies little over a piece) and end where the
+// kernels do, so that a wide r_short does not stretch them: beyond 6 eta (FP64) both are below 2e-17, beyond 5 eta
+// (FP32) below 2e-12.  Otherwise the library's functions are called.
+inline bool short_pieces(const Phys& ph) { return ph.a <= 0.5; }
+inline double short_reach(const Phys& ph, bool f64) { return fmin(ph.rs, (f64 ? 6.0 : 5.0) * ph.eta); }
 
 struct Outputs {
     double* u = nullptr;

@@ -355,3 +355,10 @@ def test_cotangent_scales_and_wide_boxes(R, scale):
     _check(one, ref, np.arange(120))
     for k in one:
         assert rel_l2(got[k] / scale, one[k]) <= GRAD_TOL
+
+
+def test_wide_short_range_radius(R):
+    """A wide r_short leaves the gradients as they are: the near part's pieces end where its kernels do."""
+    w = I.small_workload(n_atoms=70, n=(27, 19, 22), h=0.5, seed=62, ions=True, lj_rcut=4.0, net=1.0)
+    G = _cotangents(w, 31)
+    _check(_gpu_grad(R, w, G, r_short=25.0), O.grad(O.Problem.from_workload(w), np.arange(70), G["u"], G["c"], G["h"]), np.arange(70))

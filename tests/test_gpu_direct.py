@@ -212,3 +212,42 @@ def test_fp32_blocks_and_near_lists(R, n, grid, sites, mode):
     g = {k: out[k].cpu().numpy().reshape(r.S, -1) for k in keys}
     r.close()
     check_fields(g, ref, keys, 1e-6, w.grid, w.solute.xyz, label=f"{n} atoms {grid} {mode}")
+
+
+@pytest.mark.parametrize("mode", ["none", "rcut", "tol"])
+@pytest.mark.parametrize("sites", [["O", "H"], ["O", "H", "Na+", "Cl-"], ["O", "H", "Na+", "Cl-", "O", "H"]])
+@pytest.mark.parametrize("n, grid", [(1, (85, 53, 41)), (65, (85, 53, 41)), (64, (86, 49, 41)), (130, (16, 9, 5)),
+                                     (63, (15, 8, 4))])
+def test_fp64_blocks_and_tables(R, n, grid, sites, mode):
+    """The FP64 direct sum with four points per lane (a grid of at least 456 CTAs) and with one, ragged in every axis,
+    atom tiles of one source, a full one and one over, an atom on a grid point, each LJ cut-off mode and padded site
+    count.  A pair is good to a few 1e-16 and q/d - q erfc/d loses d/eta of it, a factor of 100 at the closest points."""
+    w = I.small_workload(n_atoms=n, n=grid, h=0.5, seed=72, lj_rcut=3.1 if mode == "rcut" else 0.0, net=1.0)
+    if mode == "tol":
+        w.opts["lj_tol"] = 1e-2
+    w.solvent = I.solvent(sites)
+    if n > 1:
+        w.solute.xyz[n // 2] = np.asarray(w.grid.origin) + 0.5 * np.array([grid[0] // 2, grid[1] // 2, 2])
+    keys = ("u", "c", "h") if "Na+" in sites else ("u", "c")
+    ref = O.fields(O.Problem.from_workload(w), want=keys)
+    r = R.from_workload(w, method=R.METHOD_DIRECT, precision=R.PREC_FP64)
+    out = r.init(u=True, c=True, h="h" in keys)
+    g = {k: out[k].cpu().numpy().reshape(r.S, -1) for k in keys}
+    r.close()
+    check_fields(g, ref, keys, 1e-12, w.grid, w.solute.xyz, label=f"{n} atoms {grid} {mode}")
+
+
+@pytest.mark.parametrize("kappa", [-1.0, 1.2])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_wide_short_range_radius(R, precision, kappa):
+    """The short-range pieces end where the kernels do, however wide r_short is, and a screening length of the order of
+    the smearing takes the functions themselves: the class's tolerance, which pieces 0.1 to 0.2 eta wide miss by a factor
+    of ten and more."""
+    w = I.small_workload(n_atoms=70, n=(37, 21, 13), h=0.5, seed=74, ions=True, lj_rcut=5.0, net=1.0)
+    w.opts["kappa"] = kappa
+    prec, tol = (R.PREC_FP32, 1e-6) if precision == "fp32" else (R.PREC_FP64, 1e-12)
+    r = R.from_workload(w, method=R.METHOD_DIRECT, precision=prec, r_short=25.0, kappa=kappa)
+    out = r.init()
+    g = {k: out[k].cpu().numpy().reshape(r.S, -1) for k in ("u", "c", "h")}
+    r.close()
+    check_fields(g, O.fields(O.Problem.from_workload(w)), ("u", "c", "h"), tol, w.grid, w.solute.xyz)
