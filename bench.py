@@ -757,7 +757,8 @@ def suite_kspace(args):
                           "roofline": {"bound": "alu", "unit": "FMA/s", "achieved": fma / (ms * 1e-3),
                                        "peak": fma_peak, "frac": fma / (ms * 1e-3) / fma_peak,
                                        "peak_source": f"FP32 FMA pipe, {SMS} SMs x 128 lanes at "
-                                                      f"{clk / 1e6:.0f} MHz ({src})"},
+                                                      f"{clk / 1e6:.0f} MHz ({src}); the sums run on the tensor "
+                                                      "cores, so the fraction may exceed 1"},
                           "err_sampled_rel_l2": err}), flush=True)
     r.close()
 
