@@ -615,7 +615,7 @@ static rism_status aerr(std::string& err, cudaError_t e, const char* what) {
 }
 
 // The cubic pieces of k_adj_near for the current smearing, screening, spacing and short-range radius.
-static cudaError_t near_table(AdjointState* s, const GridD& g, const Phys& ph) {
+static cudaError_t near_table(AdjointState* s, const GridD& g, const Phys& ph, cudaStream_t st) {
     const double key[4] = {ph.eta, g.h, ph.a, ph.rs};
     if (s->tab && std::memcmp(key, s->tab_key, sizeof key) == 0) return cudaSuccess;
     cudaError_t e;
@@ -644,7 +644,7 @@ static cudaError_t near_table(AdjointState* s, const GridD& g, const Phys& ph) {
                                          (float)(3.0 * (f1[q] - f0[q]) - dx * (2.0 * d0[q] + d1[q])),
                                          (float)(2.0 * (f0[q] - f1[q]) + dx * (d0[q] + d1[q])));
     }
-    if ((e = cudaMemcpy(s->tab, tab.data(), sizeof(float4) * tab.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = upload(s->tab, tab.data(), sizeof(float4) * tab.size(), st)) != cudaSuccess) return e;
     std::memcpy(s->tab_key, key, sizeof key);
     return cudaSuccess;
 }
@@ -745,7 +745,7 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
             return aerr(err, e, "adjoint site table");
         s->cap_site = (int64_t)n * t.smax;
     }
-    if ((e = near_table(s, g, ph)) != cudaSuccess) return aerr(err, e, "adjoint kernel table");
+    if ((e = near_table(s, g, ph, st)) != cudaSuccess) return aerr(err, e, "adjoint kernel table");
     SiteLJ lj;
     for (int k = 0; k < kMaxSites; ++k) {
         lj.sig[k] = k < ph.S ? sig_s[k] : 0.0;

@@ -183,7 +183,7 @@ rism_status reserve_tables(rism_ctx* c) {
             std::vector<double> tab(bytes / sizeof(double));
             if (f64) short_range_table64(ph, tab.data());
             else short_range_table(ph, c->gd.h, reinterpret_cast<float4*>(tab.data()));
-            if ((e = cudaMemcpy(c->d_sr, tab.data(), bytes, cudaMemcpyHostToDevice)) != cudaSuccess)
+            if ((e = upload(c->d_sr, tab.data(), bytes, c->st)) != cudaSuccess)
                 return cuda_fail(c, e, "short-range table");
             std::memcpy(c->sr_key, key, sizeof key);
         }
@@ -769,7 +769,7 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
             return cuda_fail(c, e, "LRA kernel table");
         std::vector<float> tab(8 * kLraTab);
         lra_table(c->ph, tab.data());
-        if ((e = cudaMemcpy(c->d_lra_tab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+        if ((e = upload(c->d_lra_tab, tab.data(), sizeof(float) * tab.size(), c->st)) != cudaSuccess)
             return cuda_fail(c, e, "LRA kernel table");
         c->lra_tab_key[0] = c->ph.eta;
         c->lra_tab_key[1] = c->ph.kappa;

@@ -83,6 +83,15 @@ cudaError_t raise_dyn_smem(F* kernel, size_t bytes) {
     return e;
 }
 
+// A small table from pageable host memory, complete in device memory when this returns.  The copy is ordered on `st`, the
+// stream of the kernels that read the table: a plain cudaMemcpy may return before the transfer from its staging buffer
+// has ended, and a non-blocking stream does not wait for the legacy stream it runs on.  Tables are uploaded when the
+// constants they depend on change, so the wait is rare.
+inline cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
 // ------------------------------------------------------------ PTX helpers
 __device__ __forceinline__ float rsqrt_approx(float x) {
     float y;

@@ -3223,7 +3223,7 @@ int sm_count() {
 
 // Host allocations for one solute (never inside a stream capture).
 rism_status tree_reserve(TreeState* s, const DevTables& t, const GridD& g, const Phys& ph, const rism_options& o,
-                         std::string& err) {
+                         cudaStream_t st, std::string& err) {
     cudaError_t e = cudaSuccess;
     const int n = (int)t.n;
     const int deg = o.degree, np = deg + 1, P3 = np * np * np;
@@ -3267,7 +3267,7 @@ rism_status tree_reserve(TreeState* s, const DevTables& t, const GridD& g, const
         s->cap_far_pts = M;
     }
     if (!s->wq) {
-        if ((e = cudaMalloc(&s->wq, 2 * sizeof(int))) || (e = cudaMemset(s->wq, 0, 2 * sizeof(int))))
+        if ((e = cudaMalloc(&s->wq, 2 * sizeof(int))) || (e = cudaMemsetAsync(s->wq, 0, 2 * sizeof(int), st)))
             return cuda_err(err, e, "work queue");
     }
     if (!s->side) {
@@ -3351,7 +3351,7 @@ rism_status tree_reserve(TreeState* s, const DevTables& t, const GridD& g, const
             return cuda_err(err, e, "kernel table");
         std::vector<float4> tab(2 * kNTab);
         short_range_table(ph, g.h, tab.data());
-        if ((e = cudaMemcpy(s->ntab, tab.data(), sizeof(float4) * 2 * kNTab, cudaMemcpyHostToDevice)) != cudaSuccess)
+        if ((e = upload(s->ntab, tab.data(), sizeof(float4) * 2 * kNTab, st)) != cudaSuccess)
             return cuda_err(err, e, "kernel table");
         std::memcpy(s->ntab_key, key, sizeof key);
         s->ntab_inv = (float)(kNTab / (ph.rs / g.h));
@@ -4164,7 +4164,7 @@ static void fixed_shape(TreeState* s, const rism_options& o) {
 rism_status tree_prepare(TreeState* s, const DevTables& t, const GridD& g, const Phys& ph, const rism_options& o,
                          cudaStream_t st, std::string& err) {
     if (!o.autotune) fixed_shape(s, o);
-    rism_status r = tree_reserve(s, t, g, ph, o, err);
+    rism_status r = tree_reserve(s, t, g, ph, o, st, err);
     if (r != RISM_OK) return r;
     r = tree_enqueue(s, t, g, ph, o, st, err);
     side_join(s, st);  // callers of the prepared tree may read every list next
@@ -4184,7 +4184,7 @@ static rism_status tree_autotune(TreeState* s, const DevTables& t, const GridD& 
             s->variant = it->second.first;
             s->leaf = it->second.second;
             s->tuned_key = key;
-            rism_status r = tree_reserve(s, t, g, ph, o, err);
+            rism_status r = tree_reserve(s, t, g, ph, o, st, err);
             return r != RISM_OK ? r : tree_enqueue(s, t, g, ph, o, st, err);
         }
     }
@@ -4199,7 +4199,7 @@ static rism_status tree_autotune(TreeState* s, const DevTables& t, const GridD& 
             for (int attempt = 0; attempt < 2; ++attempt) {
                 s->variant = v;
                 s->leaf = leaves[li];
-                rism_status r = tree_reserve(s, t, g, ph, o, err);
+                rism_status r = tree_reserve(s, t, g, ph, o, st, err);
                 if (r != RISM_OK) return r;
                 cudaEventRecord(e0, st);
                 r = tree_enqueue(s, t, g, ph, o, st, err);
@@ -4248,7 +4248,7 @@ static rism_status tree_autotune(TreeState* s, const DevTables& t, const GridD& 
         g_tune[key] = {bv, bl};
         tune_save();
     }
-    rism_status r = tree_reserve(s, t, g, ph, o, err);
+    rism_status r = tree_reserve(s, t, g, ph, o, st, err);
     return r != RISM_OK ? r : tree_enqueue(s, t, g, ph, o, st, err);
 }
 
@@ -4419,7 +4419,7 @@ rism_status tree_graph_step(TreeState* s, const DevTables& t, const GridD& g, co
     s->slabs_live = false;
     if (o.autotune && s->tuned_key != problem_class(t, g, ph, o)) return RISM_OK;  // time the candidates first
     if (!o.autotune) fixed_shape(s, o);
-    rism_status r = tree_reserve(s, t, g, ph, o, err);
+    rism_status r = tree_reserve(s, t, g, ph, o, st, err);
     if (r != RISM_OK) return r;
     const EvalArgs a = make_args(s, t, g, ph, o, out);
     const CPArgs cpa = make_cp(s);
@@ -4552,7 +4552,7 @@ rism_status batch_eval(std::vector<BatchItem>& items, const rism_options& o, cud
         it.tree->variant = variant;
         if (!o.autotune) it.tree->leaf = o.leaf;
         else it.tree->leaf = s0->leaf;
-        rism_status r = tree_reserve(it.tree, *it.t, it.g, it.ph, o, msg);
+        rism_status r = tree_reserve(it.tree, *it.t, it.g, it.ph, o, st, msg);
         if (r != RISM_OK) return r;
         args[b] = make_args(it.tree, *it.t, it.g, it.ph, o, it.o);
         off[b + 1] = off[b] + it.tree->nb;
@@ -4592,9 +4592,8 @@ rism_status batch_eval(std::vector<BatchItem>& items, const rism_options& o, cud
             (e = cudaMalloc(&bc->d_work, sizeof(int) * ((size_t)off[count] + 1))) != cudaSuccess ||
             (e = cudaMalloc(&bc->d_order, sizeof(int) * (2 * (size_t)off[count] + 1))) != cudaSuccess)
             return cuda_err(msg, e, "batch buffers");
-        if ((e = cudaMemcpy(bc->d_args, args.data(), sizeof(EvalArgs) * count, cudaMemcpyHostToDevice)) !=
-                cudaSuccess ||
-            (e = cudaMemcpy(bc->d_off, off.data(), sizeof(int) * (count + 1), cudaMemcpyHostToDevice)) != cudaSuccess)
+        if ((e = upload(bc->d_args, args.data(), sizeof(EvalArgs) * count, st)) != cudaSuccess ||
+            (e = upload(bc->d_off, off.data(), sizeof(int) * (count + 1), st)) != cudaSuccess)
             return cuda_err(msg, e, "batch upload");
         if ((e = cudaStreamCreateWithFlags(&bc->cs, cudaStreamNonBlocking)) != cudaSuccess)
             return cuda_err(msg, e, "capture stream");
