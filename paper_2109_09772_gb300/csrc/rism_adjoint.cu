@@ -619,7 +619,7 @@ static cudaError_t near_table(AdjointState* s, const GridD& g, const Phys& ph, c
     const double key[4] = {ph.eta, g.h, ph.a, ph.rs};
     if (s->tab && std::memcmp(key, s->tab_key, sizeof key) == 0) return cudaSuccess;
     cudaError_t e;
-    if (!s->tab && (e = cudaMalloc(&s->tab, sizeof(float4) * 4 * kAdjTab)) != cudaSuccess) return e;
+    if ((e = alloc_once(s->tab, 4 * kAdjTab)) != cudaSuccess) return e;
     const double a = ph.a, dx = ph.rs / ph.eta / kAdjTab, tsp = 2.0 / std::sqrt(M_PI);
     // values and slopes in x at the nodes; H0'' = 4 a^2 H0 + (8 x/sqrt(pi)) e^{-x^2}
     auto node = [&](int k, double (&f)[4], double (&d)[4]) {
@@ -664,12 +664,7 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     if (n == 0) return RISM_OK;
     const int64_t M = (int64_t)g.nx * g.ny * g.nz;
     cudaError_t e;
-    if (M > s->cap_w) {
-        cudaFree(s->w);
-        s->w = nullptr;
-        if ((e = cudaMalloc(&s->w, sizeof(float4) * M)) != cudaSuccess) return aerr(err, e, "adjoint weights");
-        s->cap_w = M;
-    }
+    if ((e = grow(s->cap_w, M, buf(s->w, M))) != cudaSuccess) return aerr(err, e, "adjoint weights");
     const int seg_per_row = (g.nx + kRowT - 1) / kRowT;
     const int nseg = seg_per_row * g.ny * g.nz;
     const int ablocks = (n + kAT * kAPT - 1) / (kAT * kAPT);
@@ -678,25 +673,13 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     chunks = max(1, min(chunks, min(nseg, 256)));
     const int tchunks = tree && o.method == RISM_METHOD_TREECODE ? tree_adjoint_chunks(n) : 0;
     const int64_t need_part = (int64_t)max(chunks, tchunks) * n * 4;
-    if (need_part > s->cap_part) {
-        cudaFree(s->part);
-        s->part = nullptr;
-        if ((e = cudaMalloc(&s->part, sizeof(double) * need_part)) != cudaSuccess) return aerr(err, e, "adjoint partials");
-        s->cap_part = need_part;
-    }
-    if ((int64_t)n * 9 > s->cap_near) {
-        cudaFree(s->near);
-        s->near = nullptr;
-        if ((e = cudaMalloc(&s->near, sizeof(double) * 9 * n)) != cudaSuccess) return aerr(err, e, "adjoint near");
-        s->cap_near = (int64_t)n * 9;
-    }
+    if ((e = grow(s->cap_part, need_part, buf(s->part, need_part))) != cudaSuccess) return aerr(err, e, "adjoint partials");
+    const int64_t need_near = (int64_t)n * 9, need_site = (int64_t)n * t.smax;
+    if ((e = grow(s->cap_near, need_near, buf(s->near, need_near))) != cudaSuccess) return aerr(err, e, "adjoint near");
+    if ((e = grow(s->cap_site, need_site, buf(s->site, need_site))) != cudaSuccess)
+        return aerr(err, e, "adjoint site table");
     const int64_t need_gu4 = g_u ? M * ((ph.S + 3) / 4) : 0;
-    if (need_gu4 > s->cap_gu4) {
-        cudaFree(s->gu4);
-        s->gu4 = nullptr;
-        if ((e = cudaMalloc(&s->gu4, sizeof(float4) * need_gu4)) != cudaSuccess) return aerr(err, e, "adjoint G_u");
-        s->cap_gu4 = need_gu4;
-    }
+    if (g_u && (e = grow(s->cap_gu4, need_gu4, buf(s->gu4, need_gu4))) != cudaSuccess) return aerr(err, e, "adjoint G_u");
     WeightCoef wc;
     const double cf[3] = {ph.k_e, -ph.beta * ph.k_e, -ph.beta * ph.k_e / (2.0 * ph.eps_r)};
     for (int q = 0; q < 3; ++q)
@@ -737,13 +720,6 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
         dim3 grid(ablocks, chunks);
         if (dh) k_adj_far<true><<<grid, kAT, 0, st>>>(fa);
         else k_adj_far<false><<<grid, kAT, 0, st>>>(fa);
-    }
-    if ((int64_t)n * t.smax > s->cap_site) {
-        cudaFree(s->site);
-        s->site = nullptr;
-        if ((e = cudaMalloc(&s->site, sizeof(float2) * (size_t)n * t.smax)) != cudaSuccess)
-            return aerr(err, e, "adjoint site table");
-        s->cap_site = (int64_t)n * t.smax;
     }
     if ((e = near_table(s, g, ph, st)) != cudaSuccess) return aerr(err, e, "adjoint kernel table");
     SiteLJ lj;

@@ -46,7 +46,7 @@ struct rism_ctx {
     DevErr* d_err = nullptr;
     DevErr* h_err = nullptr;  // pinned
     double* d_tail = nullptr;
-    void* d_sr = nullptr;  // short-range pieces of the direct sum, built for sr_key
+    double* d_sr = nullptr;  // short-range pieces of the direct sum, built for sr_key
     double sr_key[4] = {0.0, 0.0, 0.0, -1.0};
     // the solute, [n][6] x, y, z, q, sigma, eps, in page-locked host memory: uploaded as it stands (by the
     // replayed graph's copy node or an asynchronous copy); every entry point that uploads it synchronises its
@@ -55,7 +55,7 @@ struct rism_ctx {
     int64_t cap_h_raw = 0;
     double* h_tail = nullptr;  // pinned [RISM_MAX_SITES]
     double* d_stage[3] = {nullptr, nullptr, nullptr};
-    size_t stage_bytes[3] = {0, 0, 0};
+    int64_t stage_len[3] = {0, 0, 0};
     TreeState* tree = nullptr;
     AdjointState* adj = nullptr;
 
@@ -69,7 +69,7 @@ struct rism_ctx {
     cudaEvent_t cp_fork = nullptr, cp_join[3] = {nullptr, nullptr, nullptr};
     // all-space long-range integral: chunk partials, per-atom sums, totals (device) and the totals' host copy
     double* d_lra_part = nullptr;
-    size_t lra_part_cap = 0;
+    int64_t lra_part_cap = 0;
     double2* d_lra_atom = nullptr;
     int64_t lra_atom_cap = 0;
     double* d_lra_tot = nullptr;
@@ -78,17 +78,17 @@ struct rism_ctx {
     float* d_lra_tab = nullptr;   // cubic pieces of the overlap integrals for lra_tab_key = (eta, kappa)
     double lra_tab_key[2] = {0.0, -1.0};
     // the atoms in a spatial order for the pair sum (position -> original index), recomputed for a new solute
-    int* h_lra_perm = nullptr;    // pinned [lra_perm_cap]
+    int* h_lra_perm = nullptr;    // pinned [lra_hperm_cap]
     int* d_lra_perm = nullptr;
-    void* d_lra_src = nullptr;    // the sorted source table
-    int64_t lra_perm_cap = 0;
+    SrcF* d_lra_src = nullptr;    // the sorted source table
+    int64_t lra_perm_cap = 0, lra_hperm_cap = 0;
     int64_t lra_perm_version = -1;
     int64_t solute_version = 0;   // incremented by every rism_set_solute
     // reciprocal-space asymptotics: per-atom phase tables and device staging for host outputs
-    void* d_ktab = nullptr;
-    size_t ktab_bytes = 0;
+    unsigned char* d_ktab = nullptr;
+    int64_t ktab_bytes = 0;
     double* d_kstage[2] = {nullptr, nullptr};
-    size_t kstage_bytes = 0;
+    int64_t kstage_len = 0;
 };
 
 namespace {
@@ -143,28 +143,12 @@ void make_phys(rism_ctx* c) {
 rism_status reserve_tables(rism_ctx* c) {
     cudaError_t e;
     const int smax = padded_sites(c->S);
-    if (c->n > c->cap_n || smax != c->cap_smax) {
-        cudaFree(c->d_raw);
-        cudaFree(c->t.geo);
-        cudaFree(c->t.srcf);
-        cudaFree(c->t.ljd);
-        cudaFree(c->t.ljf);
-        c->d_raw = nullptr;
-        c->t.geo = nullptr;
-        c->t.srcf = nullptr;
-        c->t.ljd = nullptr;
-        c->t.ljf = nullptr;
-        c->cap_n = 0;
-        int64_t n = c->n > 0 ? c->n : 1;
-        if ((e = cudaMalloc(&c->d_raw, sizeof(double) * 6 * n)) != cudaSuccess ||
-            (e = cudaMalloc(&c->t.geo, sizeof(Geo) * n)) != cudaSuccess ||
-            (e = cudaMalloc(&c->t.srcf, sizeof(SrcF) * n)) != cudaSuccess ||
-            (e = cudaMalloc(&c->t.ljd, sizeof(LJd) * n * smax)) != cudaSuccess ||
-            (e = cudaMalloc(&c->t.ljf, sizeof(LJf) * n * smax)) != cudaSuccess)
-            return cuda_fail(c, e, "allocating solute tables");
-        c->cap_n = n;
-        c->cap_smax = smax;
-    }
+    if (smax != c->cap_smax) c->cap_n = 0;
+    const int64_t n = std::max<int64_t>(c->n, 1);
+    if ((e = grow(c->cap_n, n, buf(c->d_raw, 6 * n), buf(c->t.geo, n), buf(c->t.srcf, n), buf(c->t.ljd, n * smax),
+                  buf(c->t.ljf, n * smax))) != cudaSuccess)
+        return cuda_fail(c, e, "allocating solute tables");
+    c->cap_smax = smax;
     c->t.n = c->n;
     c->t.smax = smax;
     c->t.err = c->d_err;
@@ -179,8 +163,8 @@ rism_status reserve_tables(rism_ctx* c) {
         const double key[4] = {ph.eta, c->gd.h, ph.a, ph.rs};
         const size_t bytes = f64 ? sizeof(double) * kLen64 : sizeof(float4) * 2 * kNTab;
         if (!c->d_sr || std::memcmp(key, c->sr_key, sizeof key) != 0) {
-            if (!c->d_sr && (e = cudaMalloc(&c->d_sr, bytes)) != cudaSuccess) return cuda_fail(c, e, "short-range table");
             std::vector<double> tab(bytes / sizeof(double));
+            if ((e = alloc_once(c->d_sr, tab.size())) != cudaSuccess) return cuda_fail(c, e, "short-range table");
             if (f64) short_range_table64(ph, tab.data());
             else short_range_table(ph, c->gd.h, reinterpret_cast<float4*>(tab.data()));
             if ((e = upload(c->d_sr, tab.data(), bytes, c->st)) != cudaSuccess)
@@ -188,9 +172,9 @@ rism_status reserve_tables(rism_ctx* c) {
             std::memcpy(c->sr_key, key, sizeof key);
         }
         if (f64) {
-            c->t.sr64 = static_cast<const double*>(c->d_sr);
+            c->t.sr64 = c->d_sr;
         } else {
-            c->t.sr = static_cast<const float4*>(c->d_sr);
+            c->t.sr = reinterpret_cast<const float4*>(c->d_sr);
             c->t.sr_inv = (float)(kNTab / (ph.rs / c->gd.h));
         }
     }
@@ -288,10 +272,10 @@ rism_status rism_grid_create(const rism_grid_desc* grid, const rism_options* opt
     }
     c->st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaGetDevice(&c->device);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_err, sizeof(DevErr));
-    if (e == cudaSuccess) e = cudaMallocHost(&c->h_err, sizeof(DevErr));
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_tail, sizeof(double) * kMaxSites);
-    if (e == cudaSuccess) e = cudaMallocHost(&c->h_tail, sizeof(double) * kMaxSites);
+    if (e == cudaSuccess) e = alloc_once(c->d_err, 1);
+    if (e == cudaSuccess) e = alloc_once<PinnedMem>(c->h_err, 1);
+    if (e == cudaSuccess) e = alloc_once(c->d_tail, kMaxSites);
+    if (e == cudaSuccess) e = alloc_once<PinnedMem>(c->h_tail, kMaxSites);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(DevErr), c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     if (e != cudaSuccess) {
@@ -311,14 +295,10 @@ rism_status rism_set_solute(rism_ctx* c, int64_t n, const double* xyz, const dou
     if (!c) return RISM_E_INVALID;
     if (const char* m = check_host_solute(n, xyz, q, sigma, eps)) return fail(c, RISM_E_INVALID, m);
     if (n > c->cap_h_raw) {
-        cudaFreeHost(c->h_raw);
-        c->h_raw = nullptr;
-        c->cap_h_raw = 0;
         c->n = 0;
         c->have_solute = false;
-        const cudaError_t e = cudaMallocHost(&c->h_raw, sizeof(double) * 6 * n);
+        const cudaError_t e = grow_with<PinnedMem>(c->cap_h_raw, n, buf(c->h_raw, 6 * n));
         if (e != cudaSuccess) return cuda_fail(c, e, "page-locked solute buffer");
-        c->cap_h_raw = n;
     }
     double* raw = c->h_raw;
     for (int64_t i = 0; i < n; ++i) {
@@ -436,13 +416,8 @@ rism_status rism_init(rism_ctx* c, double* u, double* c_lr, double* h_lr, double
             // straight into page-locked host memory measured slower here than the copy engines.
             host_out = true;
             staged[k] = true;
-            if (c->stage_bytes[k] < bytes) {
-                cudaFree(c->d_stage[k]);
-                c->d_stage[k] = nullptr;
-                c->stage_bytes[k] = 0;
-                if ((e = cudaMalloc(&c->d_stage[k], bytes)) != cudaSuccess) return cuda_fail(c, e, "staging buffer");
-                c->stage_bytes[k] = bytes;
-            }
+            if ((e = grow(c->stage_len[k], (int64_t)c->S * M, buf(c->d_stage[k], (int64_t)c->S * M))) != cudaSuccess)
+                return cuda_fail(c, e, "staging buffer");
             dev[k] = c->d_stage[k];
         }
     }
@@ -736,37 +711,21 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
     int sms = 0;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess)
         return cuda_fail(c, e, "device attribute");
-    const size_t need = lra_scratch_doubles(n, sms);
-    if (need > c->lra_part_cap) {
-        cudaFree(c->d_lra_part);
-        c->d_lra_part = nullptr;
-        c->lra_part_cap = 0;
-        if ((e = cudaMalloc(&c->d_lra_part, sizeof(double) * need)) != cudaSuccess)
-            return cuda_fail(c, e, "LRA scratch");
-        c->lra_part_cap = need;
-    }
-    if (n > c->lra_atom_cap) {
-        cudaFree(c->d_lra_atom);
-        c->d_lra_atom = nullptr;
-        c->lra_atom_cap = 0;
-        if ((e = cudaMalloc(&c->d_lra_atom, sizeof(double2) * n)) != cudaSuccess)
-            return cuda_fail(c, e, "LRA atom sums");
-        c->lra_atom_cap = n;
-    }
+    const int64_t need = (int64_t)lra_scratch_doubles(n, sms);
+    if ((e = grow(c->lra_part_cap, need, buf(c->d_lra_part, need))) != cudaSuccess) return cuda_fail(c, e, "LRA scratch");
+    if ((e = grow(c->lra_atom_cap, n, buf(c->d_lra_atom, n))) != cudaSuccess) return cuda_fail(c, e, "LRA atom sums");
     if (lra_total_doubles(n) != c->lra_tot_len) {  // the counter's place depends on the length
-        cudaFree(c->d_lra_tot);
-        c->d_lra_tot = nullptr;
-        c->lra_tot_len = 0;
         const size_t len = lra_total_doubles(n);
-        if ((!c->h_lra_tot && (e = cudaMallocHost(&c->h_lra_tot, sizeof(double) * 3)) != cudaSuccess) ||
-            (e = cudaMalloc(&c->d_lra_tot, sizeof(double) * len)) != cudaSuccess ||
+        c->lra_tot_len = 0;
+        int64_t cap = 0;
+        if ((e = alloc_once<PinnedMem>(c->h_lra_tot, 3)) != cudaSuccess ||
+            (e = grow(cap, (int64_t)len, buf(c->d_lra_tot, (int64_t)len))) != cudaSuccess ||
             (e = cudaMemsetAsync(c->d_lra_tot, 0, sizeof(double) * len, c->st)) != cudaSuccess)
             return cuda_fail(c, e, "LRA totals");
         c->lra_tot_len = len;
     }
     if (!c->d_lra_tab || c->lra_tab_key[0] != c->ph.eta || c->lra_tab_key[1] != c->ph.kappa) {
-        if (!c->d_lra_tab && (e = cudaMalloc(&c->d_lra_tab, sizeof(float) * 8 * kLraTab)) != cudaSuccess)
-            return cuda_fail(c, e, "LRA kernel table");
+        if ((e = alloc_once(c->d_lra_tab, 8 * kLraTab)) != cudaSuccess) return cuda_fail(c, e, "LRA kernel table");
         std::vector<float> tab(8 * kLraTab);
         lra_table(c->ph, tab.data());
         if ((e = upload(c->d_lra_tab, tab.data(), sizeof(float) * tab.size(), c->st)) != cudaSuccess)
@@ -775,19 +734,10 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
         c->lra_tab_key[1] = c->ph.kappa;
     }
     if (n > c->lra_perm_cap) {
-        cudaFree(c->d_lra_perm);
-        cudaFree(c->d_lra_src);
-        cudaFreeHost(c->h_lra_perm);
-        c->d_lra_perm = nullptr;
-        c->d_lra_src = nullptr;
-        c->h_lra_perm = nullptr;
-        c->lra_perm_cap = 0;
         c->lra_perm_version = -1;
-        if ((e = cudaMalloc(&c->d_lra_perm, sizeof(int) * n)) != cudaSuccess ||
-            (e = cudaMalloc(&c->d_lra_src, sizeof(SrcF) * n)) != cudaSuccess ||
-            (e = cudaMallocHost(&c->h_lra_perm, sizeof(int) * n)) != cudaSuccess)
+        if ((e = grow_with<PinnedMem>(c->lra_hperm_cap, n, buf(c->h_lra_perm, n))) != cudaSuccess ||
+            (e = grow(c->lra_perm_cap, n, buf(c->d_lra_perm, n), buf(c->d_lra_src, n))) != cudaSuccess)
             return cuda_fail(c, e, "LRA atom order");
-        c->lra_perm_cap = n;
     }
     if (c->lra_perm_version != c->solute_version) {  // a new solute: its spatial order
         lra_order(c->h_raw, n, c->h_lra_perm);
@@ -796,7 +746,7 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
             return cuda_fail(c, e, "LRA atom order upload");
         c->lra_perm_version = c->solute_version;
     }
-    if ((e = launch_lra(c->t, c->gd, c->ph, sms, c->d_lra_perm, static_cast<SrcF*>(c->d_lra_src), c->d_lra_tab, c->d_lra_part,
+    if ((e = launch_lra(c->t, c->gd, c->ph, sms, c->d_lra_perm, c->d_lra_src, c->d_lra_tab, c->d_lra_part,
                         c->d_lra_atom, c->d_lra_tot, c->o.wait_limit, c->st)) != cudaSuccess)
         return cuda_fail(c, e, "LRA kernels");
     if ((e = cudaMemcpyAsync(c->h_lra_tot, c->d_lra_tot, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->st)) !=
@@ -853,29 +803,17 @@ rism_status rism_asymptotics_k(rism_ctx* c, double k_tol, double* c_k, double* h
             continue;
         }
         host = true;
-        if (c->kstage_bytes < bytes) {
-            cudaFree(c->d_kstage[0]);
-            cudaFree(c->d_kstage[1]);
-            c->d_kstage[0] = c->d_kstage[1] = nullptr;
-            c->kstage_bytes = 0;
-            if ((e = cudaMalloc(&c->d_kstage[0], bytes)) != cudaSuccess ||
-                (e = cudaMalloc(&c->d_kstage[1], bytes)) != cudaSuccess)
-                return cuda_fail(c, e, "k-space staging buffer");
-            c->kstage_bytes = bytes;
-        }
+        const int64_t len = (int64_t)(bytes / sizeof(double));
+        if ((e = grow(c->kstage_len, len, buf(c->d_kstage[0], len), buf(c->d_kstage[1], len))) != cudaSuccess)
+            return cuda_fail(c, e, "k-space staging buffer");
         dev[k] = c->d_kstage[k];
     }
     int sms = 0;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess)
         return cuda_fail(c, e, "device attribute");
     const size_t tb = kspace_table_bytes(c->n, c->g.nx, c->g.ny, c->g.nz, ks, sms);
-    if (tb > c->ktab_bytes) {
-        cudaFree(c->d_ktab);
-        c->d_ktab = nullptr;
-        c->ktab_bytes = 0;
-        if ((e = cudaMalloc(&c->d_ktab, tb)) != cudaSuccess) return cuda_fail(c, e, "k-space phase tables");
-        c->ktab_bytes = tb;
-    }
+    if ((e = grow(c->ktab_bytes, (int64_t)tb, buf(c->d_ktab, (int64_t)tb))) != cudaSuccess)
+        return cuda_fail(c, e, "k-space phase tables");
     const bool timed = (c->o.debug_flags & 2) != 0;
     if (timed) {
         if (!c->ev[0]) {

@@ -11,6 +11,7 @@
 #include <utility>
 
 #include "rism3d.h"
+#include "rism_grow.h"
 
 namespace rism {
 
@@ -81,6 +82,35 @@ cudaError_t raise_dyn_smem(F* kernel, size_t bytes) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) c = bytes;
     return e;
+}
+
+// Device and page-locked host memory.  A failed allocation is reported by its return value alone: the runtime's record of
+// it is cleared, or the error check of the next launch would report it again.
+struct DeviceMem {
+    static cudaError_t alloc(void** p, size_t bytes) {
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e;
+    }
+    static void release(void* p) { cudaFree(p); }
+};
+struct PinnedMem {
+    static cudaError_t alloc(void** p, size_t bytes) {
+        const cudaError_t e = cudaMallocHost(p, bytes);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e;
+    }
+    static void release(void* p) { cudaFreeHost(p); }
+};
+template <typename Cap, typename... T>
+cudaError_t grow(Cap& cap, int64_t need, Buf<T>... b) {
+    return grow_with<DeviceMem>(cap, need, b...);
+}
+// A buffer of fixed size, allocated when first needed.
+template <typename Mem = DeviceMem, typename T>
+cudaError_t alloc_once(T*& p, size_t count) {
+    int64_t cap = p ? 1 : 0;
+    return grow_with<Mem>(cap, 1, buf(p, (int64_t)count));
 }
 
 // A small table from pageable host memory, complete in device memory when this returns.  The copy is ordered on `st`, the

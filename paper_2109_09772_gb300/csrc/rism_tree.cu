@@ -3203,13 +3203,6 @@ rism_status cuda_err(std::string& err, cudaError_t e, const char* what) {
     return e == cudaErrorMemoryAllocation ? RISM_E_NOMEM : RISM_E_CUDA;
 }
 
-template <typename T>
-cudaError_t regrow(T*& p, size_t count) {
-    cudaFree(p);
-    p = nullptr;
-    return cudaMalloc(&p, (count > 0 ? count : 1) * sizeof(T));
-}
-
 int sm_count() {
     static int n = 0;
     if (n == 0) {
@@ -3238,23 +3231,21 @@ rism_status tree_reserve(TreeState* s, const DevTables& t, const GridD& g, const
     s->max_nodes = (int)(90LL * n / (s->leaf + 1)) + 16;
     s->max_prox = 10 * n / (P3 + 1) + 2;
     s->max_items = 10 * (n / kChunk + 1) + 2;
-    if (!s->meta) {
-        if ((e = cudaMalloc(&s->meta, sizeof(TreeMeta))) != cudaSuccess) return cuda_err(err, e, "tree meta");
-        if ((e = cudaMallocHost(&s->h_meta, sizeof(TreeMeta))) != cudaSuccess) return cuda_err(err, e, "tree meta");
-        if ((e = regrow(s->cell_start, (size_t)kMaxCells)) != cudaSuccess) return cuda_err(err, e, "cell table");
+    if ((e = alloc_once(s->meta, 1))) return cuda_err(err, e, "tree meta");
+    if (!s->h_meta) {
+        if ((e = alloc_once<PinnedMem>(s->h_meta, 1))) return cuda_err(err, e, "tree meta");
         std::memset(s->h_meta, 0, sizeof(TreeMeta));
     }
-    if (n > s->cap_n || t.smax != s->smax || s->max_nodes > s->cap_nodes || deg != s->deg) {
-        const size_t nn = n > 0 ? (size_t)n : 1;
-        if ((e = regrow(s->code, nn)) || (e = regrow(s->idx, nn)) || (e = regrow(s->code2, nn)) ||
-            (e = regrow(s->idx2, nn)) || (e = regrow(s->nodes, (size_t)s->max_nodes)) ||
-            (e = regrow(s->items, 2 * (size_t)s->max_items)) || (e = regrow(s->prox_nodes, (size_t)s->max_prox)) ||
-            (e = regrow(s->prox_items, (size_t)s->max_prox + 1)) ||
-            (e = regrow(s->part, (size_t)s->max_items * P3)) || (e = regrow(s->src, nn + (size_t)s->max_prox * P3)) ||
-            (e = regrow(s->srcf, nn + (size_t)s->max_prox * P3)) || (e = regrow(s->ljs, nn * t.smax)) ||
-            (e = regrow(s->ljs2, nn * t.smax)))
+    if ((e = alloc_once(s->cell_start, (size_t)kMaxCells))) return cuda_err(err, e, "cell table");
+    const int64_t nn = n > 0 ? n : 1, nsrc = nn + (int64_t)s->max_prox * P3;
+    if (t.smax != s->smax || s->max_nodes > s->cap_nodes || deg != s->deg) s->cap_n = 0;
+    if (nn > s->cap_n) {
+        if ((e = grow(s->cap_n, nn, buf(s->code, nn), buf(s->idx, nn), buf(s->code2, nn), buf(s->idx2, nn),
+                      buf(s->nodes, s->max_nodes), buf(s->items, 2 * (int64_t)s->max_items),
+                      buf(s->prox_nodes, s->max_prox), buf(s->prox_items, (int64_t)s->max_prox + 1),
+                      buf(s->part, (int64_t)s->max_items * P3), buf(s->src, nsrc), buf(s->srcf, nsrc),
+                      buf(s->ljs, nn * t.smax), buf(s->ljs2, nn * t.smax))))
             return cuda_err(err, e, "tree buffers");
-        s->cap_n = (int64_t)nn;
         s->cap_nodes = s->max_nodes;
         s->cap_prox = s->max_prox;
         s->cap_items = s->max_items;
@@ -3262,38 +3253,27 @@ rism_status tree_reserve(TreeState* s, const DevTables& t, const GridD& g, const
         s->deg = deg;
     }
     const int64_t M = far_points(g.nx, g.ny, g.nz);
-    if (M > s->cap_far_pts) {
-        if ((e = regrow(s->far, (size_t)M))) return cuda_err(err, e, "far-field buffer");
-        s->cap_far_pts = M;
-    }
+    if ((e = grow(s->cap_far_pts, M, buf(s->far, M)))) return cuda_err(err, e, "far-field buffer");
     if (!s->wq) {
-        if ((e = cudaMalloc(&s->wq, 2 * sizeof(int))) || (e = cudaMemsetAsync(s->wq, 0, 2 * sizeof(int), st)))
+        if ((e = alloc_once(s->wq, 2))) return cuda_err(err, e, "work queue");
+        if ((e = cudaMemsetAsync(s->wq, 0, 2 * sizeof(int), st))) {
+            cudaFree(s->wq);
+            s->wq = nullptr;
             return cuda_err(err, e, "work queue");
+        }
     }
-    if (!s->side) {
-        if ((e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking)) ||
-            (e = cudaEventCreateWithFlags(&s->side_fork[0], cudaEventDisableTiming)) ||
-            (e = cudaEventCreateWithFlags(&s->side_fork[1], cudaEventDisableTiming)) ||
-            (e = cudaEventCreateWithFlags(&s->side_join, cudaEventDisableTiming)))
-            return cuda_err(err, e, "side stream");
-    }
-    if (s->nb + 1 > s->cap_nb) {
-        if ((e = regrow(s->far_cnt, (size_t)s->nb + 1)) || (e = regrow(s->near_cnt, (size_t)s->nb + 1)) ||
-            (e = regrow(s->near_work, (size_t)s->nb + 1)) || (e = regrow(s->near_order, (size_t)s->nb + 1)) ||
-            (e = regrow(s->far_work, (size_t)s->nb + 1)) || (e = regrow(s->far_order, (size_t)s->nb + 1)))
-            return cuda_err(err, e, "list counts");
-        s->cap_nb = s->nb + 1;
-    }
+    if (!s->side && (e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking))) return cuda_err(err, e, "side stream");
+    for (cudaEvent_t* ev : {&s->side_fork[0], &s->side_fork[1], &s->side_join})
+        if (!*ev && (e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming))) return cuda_err(err, e, "side stream");
+    const int64_t nb = (int64_t)s->nb + 1;
+    if ((e = grow(s->cap_nb, nb, buf(s->far_cnt, nb), buf(s->near_cnt, nb), buf(s->near_work, nb), buf(s->near_order, nb),
+                  buf(s->far_work, nb), buf(s->far_order, nb))))
+        return cuda_err(err, e, "list counts");
     if (s->cap_far == 0) s->cap_far = 128;
     if (s->cap_near == 0) s->cap_near = 512;
-    if ((int64_t)s->nb * s->cap_far > s->cap_far_ent) {
-        if ((e = regrow(s->far_ent, (size_t)s->nb * s->cap_far))) return cuda_err(err, e, "far list");
-        s->cap_far_ent = (int64_t)s->nb * s->cap_far;
-    }
-    if ((int64_t)s->nb * s->cap_near > s->cap_near_ent) {
-        if ((e = regrow(s->near_ent, (size_t)s->nb * s->cap_near))) return cuda_err(err, e, "near list");
-        s->cap_near_ent = (int64_t)s->nb * s->cap_near;
-    }
+    const int64_t nfar = (int64_t)s->nb * s->cap_far, nnear = (int64_t)s->nb * s->cap_near;
+    if ((e = grow(s->cap_far_ent, nfar, buf(s->far_ent, nfar)))) return cuda_err(err, e, "far list");
+    if ((e = grow(s->cap_near_ent, nnear, buf(s->near_ent, nnear)))) return cuda_err(err, e, "near list");
     // target boxes: levels of aligned 16 << l cubes up to one that covers the grid
     TBoxes& tb = s->tb;
     tb = TBoxes{};
@@ -3322,33 +3302,19 @@ rism_status tree_reserve(TreeState* s, const DevTables& t, const GridD& g, const
     if (tb.enabled) {
         if (s->cap_cp == 0) s->cap_cp = 64;
         if (s->cap_dn == 0) s->cap_dn = 128;
-        if (tb.nbox + 1 > s->cap_tbox) {
-            if ((e = regrow(s->cp_cnt, (size_t)tb.nbox + 1)) || (e = regrow(s->dn_cnt, (size_t)tb.nbox + 1)) ||
-                (e = regrow(s->tflag, (size_t)tb.nbox + 1)) || (e = regrow(s->tnch, (size_t)tb.nbox + 1)) ||
-                (e = regrow(s->cp_work, (size_t)tb.nbox + 1)) || (e = regrow(s->cp_order, (size_t)tb.nbox + 1)))
-                return cuda_err(err, e, "target boxes");
-            s->cap_tbox = tb.nbox + 1;
-        }
-        if ((int64_t)tb.nbox * s->cap_cp > s->cap_cp_ent) {
-            if ((e = regrow(s->cp_ent, (size_t)tb.nbox * s->cap_cp))) return cuda_err(err, e, "box lists");
-            s->cap_cp_ent = (int64_t)tb.nbox * s->cap_cp;
-        }
-        if ((int64_t)tb.nbox * s->cap_dn > s->cap_dn_ent) {
-            if ((e = regrow(s->dn_ent, (size_t)tb.nbox * s->cap_dn))) return cuda_err(err, e, "pass-down lists");
-            s->cap_dn_ent = (int64_t)tb.nbox * s->cap_dn;
-        }
-        if ((int64_t)tb.nbox * P3 > s->cap_tpot) {
-            if ((e = regrow(s->tpot, (size_t)tb.nbox * P3)) ||
-                (e = regrow(s->tpart, (size_t)tb.nbox * (kCPChunks - 1) * P3)))
-                return cuda_err(err, e, "proxy targets");
-            s->cap_tpot = (int64_t)tb.nbox * P3;
-        }
+        const int64_t nbox = tb.nbox, ncp = nbox * s->cap_cp, ndn = nbox * s->cap_dn, npot = nbox * P3;
+        if ((e = grow(s->cap_tbox, nbox + 1, buf(s->cp_cnt, nbox + 1), buf(s->dn_cnt, nbox + 1), buf(s->tflag, nbox + 1),
+                      buf(s->tnch, nbox + 1), buf(s->cp_work, nbox + 1), buf(s->cp_order, nbox + 1))))
+            return cuda_err(err, e, "target boxes");
+        if ((e = grow(s->cap_cp_ent, ncp, buf(s->cp_ent, ncp)))) return cuda_err(err, e, "box lists");
+        if ((e = grow(s->cap_dn_ent, ndn, buf(s->dn_ent, ndn)))) return cuda_err(err, e, "pass-down lists");
+        if ((e = grow(s->cap_tpot, npot, buf(s->tpot, npot), buf(s->tpart, (kCPChunks - 1) * npot))))
+            return cuda_err(err, e, "proxy targets");
     }
     // short-range kernels of the near field
     const double key[4] = {ph.eta, g.h, ph.a, ph.rs};
     if (!s->ntab || std::memcmp(key, s->ntab_key, sizeof key) != 0) {
-        if (!s->ntab && (e = cudaMalloc(&s->ntab, sizeof(float4) * 2 * kNTab)) != cudaSuccess)
-            return cuda_err(err, e, "kernel table");
+        if ((e = alloc_once(s->ntab, 2 * kNTab))) return cuda_err(err, e, "kernel table");
         std::vector<float4> tab(2 * kNTab);
         short_range_table(ph, g.h, tab.data());
         if ((e = upload(s->ntab, tab.data(), sizeof(float4) * 2 * kNTab, st)) != cudaSuccess)
@@ -4586,11 +4552,9 @@ rism_status batch_eval(std::vector<BatchItem>& items, const rism_options& o, cud
     if (!bc || bc->sig != sig) {
         delete bc;
         bc = new BatchCache();
-        if ((e = cudaMalloc(&bc->d_args, sizeof(EvalArgs) * count)) != cudaSuccess ||
-            (e = cudaMalloc(&bc->d_off, sizeof(int) * (count + 1))) != cudaSuccess ||
-            (e = cudaMalloc(&bc->d_queue, sizeof(int) * 2)) != cudaSuccess ||
-            (e = cudaMalloc(&bc->d_work, sizeof(int) * ((size_t)off[count] + 1))) != cudaSuccess ||
-            (e = cudaMalloc(&bc->d_order, sizeof(int) * (2 * (size_t)off[count] + 1))) != cudaSuccess)
+        if ((e = alloc_once(bc->d_args, count)) || (e = alloc_once(bc->d_off, count + 1)) ||
+            (e = alloc_once(bc->d_queue, 2)) || (e = alloc_once(bc->d_work, (size_t)off[count] + 1)) ||
+            (e = alloc_once(bc->d_order, 2 * (size_t)off[count] + 1)))
             return cuda_err(msg, e, "batch buffers");
         if ((e = upload(bc->d_args, args.data(), sizeof(EvalArgs) * count, st)) != cudaSuccess ||
             (e = upload(bc->d_off, off.data(), sizeof(int) * (count + 1), st)) != cudaSuccess)
@@ -5324,37 +5288,19 @@ rism_status tree_adjoint_far(TreeState* s, const DevTables& t, const GridD& g, c
     const int nb0 = tb.nbx[0] * tb.nby[0] * tb.nbz[0];
     // upper bound of the target groups: every leaf adds at most one partial group (the count stays on the device)
     const int nleaf = n / kAL + s->max_nodes + 1;
-    auto grow = [&](auto*& p, int64_t& cap, int64_t need) -> cudaError_t {
-        if (need <= cap) return cudaSuccess;
-        cudaFree(p);
-        p = nullptr;
-        cap = 0;
-        cudaError_t r = cudaMalloc(&p, sizeof(*p) * (size_t)need);
-        if (r == cudaSuccess) cap = need;
-        return r;
-    };
-    if ((e = grow(A.qpart, A.cap_qpart, (int64_t)nb0 * tb.P3)) != cudaSuccess ||
-        (e = grow(A.qtot, A.cap_qtot, (int64_t)tb.nbox * tb.P3)) != cudaSuccess ||
-        (e = grow(A.rlow, A.cap_rlow, (int64_t)nb0)) != cudaSuccess)
+    const int64_t nqp = (int64_t)nb0 * tb.P3, nqt = (int64_t)tb.nbox * tb.P3, ngrp = (int64_t)nleaf + 1;
+    if ((e = grow(A.cap_qpart, nqp, buf(A.qpart, nqp))) || (e = grow(A.cap_qtot, nqt, buf(A.qtot, nqt))) ||
+        (e = grow(A.cap_rlow, nb0, buf(A.rlow, nb0))))
         return cuda_err(err, e, "reverse-mode box buffers");
-    if (!A.meta) {
-        if ((e = cudaMalloc(&A.meta, sizeof(AdjTreeMeta))) != cudaSuccess ||
-            (e = cudaMallocHost(&A.h_meta, sizeof(AdjTreeMeta))) != cudaSuccess ||
-            (e = cudaMalloc(&A.nleaf, sizeof(int))) != cudaSuccess)
-            return cuda_err(err, e, "reverse-mode meta");
-    }
-    if ((e = grow(A.grp, A.cap_grp, (int64_t)nleaf + 1)) != cudaSuccess)
-        return cuda_err(err, e, "reverse-mode leaves");
+    if ((e = alloc_once(A.meta, 1)) || (e = alloc_once<PinnedMem>(A.h_meta, 1)) || (e = alloc_once(A.nleaf, 1)))
+        return cuda_err(err, e, "reverse-mode meta");
+    if ((e = grow(A.cap_grp, ngrp, buf(A.grp, ngrp)))) return cuda_err(err, e, "reverse-mode leaves");
     k_leaf_list<<<1, 1024, 0, st>>>(s->meta, s->nodes, A.grp, A.nleaf);
     launch_adj_q_deg(tb, w, A.qpart, A.rlow, A.qtot, st);
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if (nleaf + 1 > A.cap_leaf) {
-            cudaFree(A.cnt);
-            A.cnt = nullptr;
-            if ((e = cudaMalloc(&A.cnt, sizeof(int) * (nleaf + 1))) != cudaSuccess) return cuda_err(err, e, "lists");
-            A.cap_leaf = nleaf + 1;
-        }
-        if ((e = grow(A.ent, A.cap_ent, (int64_t)nleaf * A.cap)) != cudaSuccess) return cuda_err(err, e, "lists");
+        const int64_t nent = (int64_t)nleaf * A.cap;
+        if ((e = grow(A.cap_leaf, ngrp, buf(A.cnt, ngrp))) || (e = grow(A.cap_ent, nent, buf(A.ent, nent))))
+            return cuda_err(err, e, "lists");
         cudaMemsetAsync(A.meta, 0, sizeof(AdjTreeMeta), st);
         k_adj_lists<<<(nleaf + kListWarps - 1) / kListWarps, 32 * kListWarps, 0, st>>>(
             tb, s->srcf, A.grp, A.nleaf, (float)o.theta, A.cap, A.cnt, A.ent, A.meta);

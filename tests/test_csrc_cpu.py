@@ -3,6 +3,7 @@ with the system compiler and run here."""
 import glob
 import os
 import re
+import subprocess
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2109_09772_gb300", "csrc")
@@ -25,3 +26,71 @@ def test_every_copy_names_its_stream():
     bad = [f"{name}: {m.group(0)}" for name, s in _code().items()
            for m in re.finditer(r"\bcudaMem(cpy|cpy2D|cpy3D|cpyToSymbol|cpyFromSymbol|set|set2D)\s*\(", s)]
     assert not bad, bad
+
+
+GROW = r"""
+#include <assert.h>
+#include <stdlib.h>
+#include <vector>
+#include "rism_grow.h"
+static long budget;  // bytes the allocator still gives
+static int allocs, live;
+struct Host {
+    static int alloc(void** p, size_t n) {
+        ++allocs;
+        if ((long)n > budget) return 2;
+        budget -= (long)n, ++live;
+        *p = malloc(n);
+        return 0;
+    }
+    static void release(void* p) { if (p) --live; free(p); }
+};
+using namespace rism;
+int main() {
+    double* a = nullptr;
+    int* b = nullptr;
+    int64_t cap = 0;
+    budget = 10000;
+    assert(grow_with<Host>(cap, 100, buf(a, 100), buf(b, 200)) == 0 && cap == 100 && a && b && live == 2);
+    a[99] = 1.0, b[199] = 1;
+    // a smaller or equal need keeps the buffers
+    allocs = 0;
+    double* a0 = a;
+    assert(grow_with<Host>(cap, 7, buf(a, 7), buf(b, 14)) == 0 && grow_with<Host>(cap, 100, buf(a, 100), buf(b, 200)) == 0);
+    assert(allocs == 0 && a == a0 && cap == 100);
+    // the first, then the second allocation of the group fails: the capacity is gone with the pointers
+    for (int second = 0; second < 2; ++second) {
+        budget = second ? 8 * 1000 : 100;
+        assert(grow_with<Host>(cap, 1000, buf(a, 1000), buf(b, 2000)) == 2 && cap == 0 && !b);
+        assert(!a == !second);
+        // ... so a smaller need than the one the group held before allocates again
+        budget = 10000;
+        allocs = 0;
+        assert(grow_with<Host>(cap, 50, buf(a, 50), buf(b, 100)) == 0 && cap == 50 && allocs == 2 && a && b && live == 2);
+        a[49] = 1.0, b[99] = 1;
+    }
+    // an int capacity, and a need of nothing still gives a buffer
+    char* c = nullptr;
+    int icap = 0;
+    assert(grow_with<Host>(icap, 0, buf(c, 0)) == 0 && icap == 1 && c);
+    c[0] = 1;
+    Host::release(a), Host::release(b), Host::release(c);
+    assert(live == 0);
+    return 0;
+}
+"""
+
+
+def test_a_failed_allocation_leaves_no_capacity(tmp_path):
+    src, exe = tmp_path / "grow.cpp", tmp_path / "grow"
+    src.write_text(GROW)
+    subprocess.check_call(["g++", "-std=c++17", "-Wall", "-I", CSRC, str(src), "-o", str(exe)])
+    subprocess.check_call([str(exe)])
+
+
+def test_every_buffer_goes_through_the_grow_helper():
+    """A capacity kept across a failed allocation lets the next, smaller call launch kernels on null pointers: only the
+    helper allocates (rism_internal.cuh holds its two allocators)."""
+    for name, s in _code().items():
+        n = len(re.findall(r"\bcudaMalloc(Host|Async|Managed)?\s*\(", s))
+        assert n == (2 if name == "rism_internal.cuh" else 0), (name, n)
