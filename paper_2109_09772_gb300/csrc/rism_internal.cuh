@@ -44,8 +44,10 @@ struct __align__(16) LJf {
 // grid origin as float-float (hi + lo, |lo| <= ulp(hi)/2) and charge.  Grid
 // point indices are exact small integers in FP32, so for a nearby source
 // dx = (i - xh) - xl loses nothing in the first subtraction (Sterbenz) and
-// carries one rounding of dx itself.  on_grid = 1 when the source sits
-// exactly on a lattice point (only then can d = 0 occur).
+// carries one rounding of dx itself.  on_grid = 1 when the source sits on a
+// lattice point; only then can d^2 be 0, and it is never a subnormal number
+// (whose approximate reciprocal root is infinite): a source that close to a
+// lattice point is put on it (make_srcf).
 struct __align__(16) SrcF {
     float xh, yh, zh, q;
     float xl, yl, zl, on_grid;
@@ -310,13 +312,24 @@ __device__ __forceinline__ void split_ff(double v, float& hi, float& lo) {
     lo = __double2float_rn(v - (double)hi);
 }
 
+// d^2 (grid units) from a lattice point below which a source counts as being on it: FP32's smallest normal number, with
+// room for the rounding of d^2.  Only coordinates next to lattice index 0 resolve such distances.
+constexpr double kOnGrid2 = 1.18e-38;
 __device__ __forceinline__ SrcF make_srcf(double x, double y, double z, double q) {
     SrcF s;
+    const double ix = rint(x), iy = rint(y), iz = rint(z);
+    const double dx = x - ix, dy = y - iy, dz = z - iz;
+    s.on_grid = 0.f;
+    if (dx * dx + dy * dy + dz * dz < kOnGrid2) {
+        x = ix;
+        y = iy;
+        z = iz;
+        s.on_grid = 1.f;
+    }
     split_ff(x, s.xh, s.xl);
     split_ff(y, s.yh, s.yl);
     split_ff(z, s.zh, s.zl);
     s.q = (float)q;
-    s.on_grid = (x == floor(x) && y == floor(y) && z == floor(z)) ? 1.f : 0.f;
     return s;
 }
 

@@ -251,3 +251,25 @@ def test_wide_short_range_radius(R, precision, kappa):
     g = {k: out[k].cpu().numpy().reshape(r.S, -1) for k in ("u", "c", "h")}
     r.close()
     check_fields(g, O.fields(O.Problem.from_workload(w)), ("u", "c", "h"), tol, w.grid, w.solute.xyz)
+
+
+@pytest.mark.parametrize("offset", [1e-30, 1e-21])
+@pytest.mark.parametrize("method", ["DIRECT", "TREECODE"])
+@pytest.mark.parametrize("grid", [(163, 117, 61), (16, 9, 5)])
+def test_atom_a_hair_from_a_grid_point(R, grid, method, offset):
+    """An atom so close to a grid point that its squared distance (in grid units) is zero in FP32, or below FP32's normal
+    numbers, without being on it: c and h take their finite limits there, u is infinite, the other points are as always."""
+    w = I.small_workload(n_atoms=70, n=grid, h=0.5, seed=77, ions=True, lj_rcut=4.0, net=1.0)
+    w.grid.origin = (0.0, 0.0, 0.0)
+    w.solute.xyz += 0.25 * np.array(grid)
+    w.solute.xyz[41] = [offset, 0.0, 0.0]
+    ref = O.fields(O.Problem.from_workload(w))
+    r = R.from_workload(w, method=getattr(R, "METHOD_" + method), precision=R.PREC_FP32)
+    out = r.init()
+    g = {k: out[k].cpu().numpy().reshape(r.S, -1) for k in ("u", "c", "h")}
+    r.close()
+    assert np.all(np.isinf(g["u"][:, 0]))
+    tol = 1e-6 if method == "DIRECT" else 1e-5
+    check_fields(g, ref, ("c", "h"), tol, w.grid, w.solute.xyz, label=f"{method} {grid}")
+    rest = np.arange(1, w.grid.npts)
+    check_fields({"u": g["u"][:, 1:]}, {"u": ref["u"][:, 1:]}, ("u",), tol, w.grid, w.solute.xyz, idx=rest)
