@@ -253,6 +253,7 @@ struct NearAdjArgs {
     const float4* tab;       // [kAdjTab][4]: cubic pieces of C0, C1, H0, H1
     float tab_inv;           // kAdjTab / r_short (grid units)
     float rs, rs2;           // r_short (grid units)
+    float xs, aa;            // h / eta and kappa eta / 2, where the functions are called
     int wpa;                 // warps per atom: 1, 2, 4 or 8
     double* out;             // [n][9]: dq, Gx, Gy, Gz (grid units as in the far part), dLJ/dR (3), dsigma, deps
 };
@@ -277,11 +278,21 @@ __global__ void k_adj_sites(int n, int S, int smax, const double* __restrict__ r
     site[t] = v;
 }
 
-// The short-range kernels of the reverse mode in d over [0, r_short], kAdjTab cubic Hermite pieces each (built in FP64;
-// within 1e-8 of the functions, below FP32 rounding): with x = d/eta, C0 = erfc(x) and H0 = e^{-x^2}[erfcx(x-a) +
-// erfcx(x+a)] the potentials are Sc = C0/d and Sh = H0/d, and with C1 = C0 - d C0', H1 = H0 - d H0' their slopes are
-// -C1/d^2 and -H1/d^2.
+// The short-range kernels of the reverse mode in d over [0, r_short], kAdjTab cubic Hermite pieces each (built in FP64):
+// with x = d/eta, C0 = erfc(x) and H0 = e^{-x^2}[erfcx(x-a) + erfcx(x+a)] the potentials are Sc = C0/d and Sh = H0/d, and
+// with C1 = C0 - d C0', H1 = H0 - d H0' their slopes are -C1/d^2 and -H1/d^2.  Evaluated in FP32 the pieces are within 7e-8
+// (C) and 1.2e-7 (H at a = 0) to 5.5e-7 (a = 1) of the functions, which evaluated in FP32 are within 1.1e-7 and 2.7e-7 to
+// 1.0e-6; but the error of a piece grows with the fourth power of a times its width (H1 at a = 2: 1.1e-4 against 3.4e-5),
+// so a stronger screening than kAdjPieceA takes the functions.
 constexpr int kAdjTab = 256;
+constexpr double kAdjPieceA = 1.0;
+
+// C0, C1, H0, H1 at d = x eta by the functions themselves.
+__device__ __forceinline__ float4 near_functions(float x, float a) {
+    const float ex = __expf(-x * x), em = erfcxf(x - a), ep = erfcxf(x + a), c0 = erfcf(x), h0 = ex * (em + ep);
+    const float tsp = 1.12837917f;  // 2/sqrt(pi)
+    return make_float4(c0, fmaf(x * tsp, ex, c0), h0, h0 - x * (2.f * a * ex * (ep - em) - 2.f * tsp * ex));
+}
 
 struct FFs {
     float h, l;
@@ -356,18 +367,20 @@ __device__ __forceinline__ bool point_box(const GridD& g, const SrcF& sf, float 
 // terms within the largest cut-off of the atom's sites.  A lane owns a column of a tile and goes down its chord, so x
 // and y offsets are fixed and the x, y forces take the column's sum once.  Per site the sums of G_u/d^12 and G_u/d^6
 // are kept (two sites per two-wide instruction); sigma and eps gradients follow from them at the end.  FP32 sums of one
-// column, folded into float pairs per tile.  UNI: one cut-off for all of an atom's sites.
+// column, folded into float pairs per tile.  UNI: one cut-off for all of an atom's sites.  FN: the short-range kernels by
+// their functions instead of the pieces.
 // Bound by issue and the latency of the cotangent loads (two CTAs per SM at 118 registers; three at 80 spill and are
 // slower).  2,000 atoms on 128^3: 0.34 ms (1.02 ms with one CTA per atom that called erfc, erfcx and, in every thread,
 // the FP64 mixing derivatives); 55,000 atoms on 320x320x384, u and c: 7.7 ms (21.2).
-template <int NR, bool UNI>
+template <int NR, bool UNI, bool FN>
 __global__ void __launch_bounds__(kNearT) k_adj_near(const __grid_constant__ NearAdjArgs a) {
     __shared__ float4 tab[kAdjTab][4];
     __shared__ FFs red[kNearT / 32][9];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const GridD& g = a.g;
     const int64_t plane = (int64_t)g.nx * g.ny, M = plane * g.nz;
-    for (int k = threadIdx.x; k < 4 * kAdjTab; k += kNearT) tab[k >> 2][k & 3] = a.tab[k];
+    if (!FN)
+        for (int k = threadIdx.x; k < 4 * kAdjTab; k += kNearT) tab[k >> 2][k & 3] = a.tab[k];
     __syncthreads();
     const int per = (kNearT / 32) / a.wpa, sub = w % a.wpa;  // atoms per CTA pass; this warp's share of its atom
     for (int p0 = blockIdx.x * per; p0 < a.n; p0 += gridDim.x * per) {
@@ -393,17 +406,27 @@ __global__ void __launch_bounds__(kNearT) k_adj_near(const __grid_constant__ Nea
                     const float d2 = fmaf(dz, dz, c.dxy2);
                     const bool ok = d2 < a.rs2 && d2 > 0.f;
                     const float dd = ok ? d2 : 1.f;
-                    const float ri = rsqrt_approx(dd), u = dd * ri * a.tab_inv;
-                    // segment of u: adding 1.5 2^23 leaves round(u - 1/2) in the low bits of the sum
-                    const float sh = (u - 0.5f) + 12582912.0f;
-                    const int it = min(__float_as_int(sh) - 0x4B400000, kAdjTab - 1);
-                    const float tt = u - fminf(sh - 12582912.0f, (float)(kAdjTab - 1));
-                    auto piece = [&](int f) {
-                        const float4 k = tab[it][f];
-                        return fmaf(fmaf(fmaf(k.w, tt, k.z), tt, k.y), tt, k.x);
-                    };
+                    const float ri = rsqrt_approx(dd);
                     const float wc = ok ? W.x : 0.f, wh = ok ? W.y : 0.f;
-                    const float f0 = fmaf(wc, piece(0), wh * piece(2)), f1 = fmaf(wc, piece(1), wh * piece(3));
+                    float f0, f1;
+                    if (FN) {
+                        const float4 k = near_functions(dd * ri * a.xs, a.aa);
+                        // without a cotangent of h nothing of its kernel enters (it overflows at extreme screening)
+                        f0 = fmaf(wc, k.x, wh != 0.f ? wh * k.z : 0.f);
+                        f1 = fmaf(wc, k.y, wh != 0.f ? wh * k.w : 0.f);
+                    } else {
+                        const float u = dd * ri * a.tab_inv;
+                        // segment of u: adding 1.5 2^23 leaves round(u - 1/2) in the low bits of the sum
+                        const float sh = (u - 0.5f) + 12582912.0f;
+                        const int it = min(__float_as_int(sh) - 0x4B400000, kAdjTab - 1);
+                        const float tt = u - fminf(sh - 12582912.0f, (float)(kAdjTab - 1));
+                        auto piece = [&](int f) {
+                            const float4 k = tab[it][f];
+                            return fmaf(fmaf(fmaf(k.w, tt, k.z), tt, k.y), tt, k.x);
+                        };
+                        f0 = fmaf(wc, piece(0), wh * piece(2));
+                        f1 = fmaf(wc, piece(1), wh * piece(3));
+                    }
                     dq = fmaf(-f0, ri, dq);
                     const float rad = f1 * ri * ri * ri;
                     rs += rad;
@@ -548,6 +571,17 @@ __global__ void __launch_bounds__(kNearT) k_adj_near(const __grid_constant__ Nea
     }
 }
 
+template <bool FN>
+void near_launch(const NearAdjArgs& a, int S, bool uni, int ctas, cudaStream_t st) {
+    if (S <= 4) {
+        if (uni) k_adj_near<1, true, FN><<<ctas, kNearT, 0, st>>>(a);
+        else k_adj_near<1, false, FN><<<ctas, kNearT, 0, st>>>(a);
+    } else {
+        if (uni) k_adj_near<2, true, FN><<<ctas, kNearT, 0, st>>>(a);
+        else k_adj_near<2, false, FN><<<ctas, kNearT, 0, st>>>(a);
+    }
+}
+
 struct FinalArgs {
     int n, chunks;
     double h;
@@ -657,9 +691,10 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
         err = "the adjoint is implemented with FP32 pair terms (precision RISM_PREC_FP32)";
         return RISM_E_UNSUPPORTED;
     }
-    // the short-range kernels end at (5 + a) eta for FP32 (2e-12 of the whole): a wider r_short does not stretch the pieces
+    // the short-range kernels end at (5 + a) eta for FP32 (3e-12 of the whole): a wider r_short does not stretch the pieces
     Phys ph = ph_;
-    ph.rs = std::min(ph.rs, (5.0 + ph.a) * ph.eta);
+    const bool pieces = ph.a <= kAdjPieceA;
+    if (pieces) ph.rs = std::min(ph.rs, (5.0 + ph.a) * ph.eta);
     const int n = (int)t.n;
     if (n == 0) return RISM_OK;
     const int64_t M = (int64_t)g.nx * g.ny * g.nz;
@@ -721,7 +756,7 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
         if (dh) k_adj_far<true><<<grid, kAT, 0, st>>>(fa);
         else k_adj_far<false><<<grid, kAT, 0, st>>>(fa);
     }
-    if ((e = near_table(s, g, ph, st)) != cudaSuccess) return aerr(err, e, "adjoint kernel table");
+    if (pieces && (e = near_table(s, g, ph, st)) != cudaSuccess) return aerr(err, e, "adjoint kernel table");
     SiteLJ lj;
     for (int k = 0; k < kMaxSites; ++k) {
         lj.sig[k] = k < ph.S ? sig_s[k] : 0.0;
@@ -741,6 +776,8 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     na.order = (tree && o.method == RISM_METHOD_TREECODE) ? tree_atom_order(tree) : nullptr;
     na.tab = s->tab;
     na.tab_inv = (float)(kAdjTab / (ph.rs / g.h));
+    na.xs = (float)(g.h / ph.eta);
+    na.aa = (float)ph.a;
     na.rs = (float)(ph.rs / g.h);
     na.rs2 = (float)((ph.rs / g.h) * (ph.rs / g.h));
     na.out = s->near;
@@ -749,13 +786,8 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     while (na.wpa < kNearT / 32 && (int64_t)n * na.wpa < 64 * 152) na.wpa *= 2;
     const int nctas = (int)std::min<int64_t>(((int64_t)n * na.wpa + kNearT / 32 - 1) / (kNearT / 32), 4 * 152);
     const bool uni = o.lj_mode != RISM_LJ_TOL;
-    if (ph.S <= 4) {
-        if (uni) k_adj_near<1, true><<<nctas, kNearT, 0, st>>>(na);
-        else k_adj_near<1, false><<<nctas, kNearT, 0, st>>>(na);
-    } else {
-        if (uni) k_adj_near<2, true><<<nctas, kNearT, 0, st>>>(na);
-        else k_adj_near<2, false><<<nctas, kNearT, 0, st>>>(na);
-    }
+    if (pieces) near_launch<false>(na, ph.S, uni, nctas, st);
+    else near_launch<true>(na, ph.S, uni, nctas, st);
     FinalArgs fin{n, chunks, g.h, raw_dev, s->part, s->near, d_xyz, d_q, d_sigma, d_eps};
     k_adj_final<<<(n + 255) / 256, 256, 0, st>>>(fin);
     if ((e = cudaGetLastError()) != cudaSuccess) return aerr(err, e, "adjoint kernels");

@@ -33,8 +33,8 @@ void short_range_table(const Phys& ph, double h, float4* tab);
 constexpr int kTab64 = 256, kTerm64 = 8, kLen64 = 2 * kTab64 * kTerm64 + 512;
 void short_range_table64(const Phys& ph, double* tab);
 // The pieces serve the direct sum for a = kappa eta/2 up to 1/2 (e^{-2ax} varies little over a piece) and end where the
-// kernels do, so that a wide r_short does not stretch them: beyond 6 eta (FP64) both are below 2e-17, beyond 5 eta
-// (FP32) below 2e-12.  Otherwise the library's functions are called.
+// kernels do, so that a wide r_short does not stretch them: beyond 6 eta (FP64) F_c is below 2.2e-17 and F_h below
+// 4.4e-17, beyond 5 eta (FP32) below 1.6e-12 and 3.2e-12.  Otherwise the library's functions are called.
 inline bool short_pieces(const Phys& ph) { return ph.a <= 0.5; }
 inline double short_reach(const Phys& ph, bool f64) { return fmin(ph.rs, (f64 ? 6.0 : 5.0) * ph.eta); }
 

@@ -362,3 +362,42 @@ def test_wide_short_range_radius(R):
     w = I.small_workload(n_atoms=70, n=(27, 19, 22), h=0.5, seed=62, ions=True, lj_rcut=4.0, net=1.0)
     G = _cotangents(w, 31)
     _check(_gpu_grad(R, w, G, r_short=25.0), O.grad(O.Problem.from_workload(w), np.arange(70), G["u"], G["c"], G["h"]), np.arange(70))
+
+
+@pytest.mark.parametrize("method", ["DIRECT", "TREECODE"])
+@pytest.mark.parametrize("kappa", [1.0, 2.0, 4.0, 8.0])
+def test_strong_screening_near_terms(R, kappa, method):
+    """One grid point with a cotangent of h, 600 unit charges at distances of 0.02 to 7 A from it: every atom's charge and
+    position gradient is one value of the TCF kernel and of its slope, at screening lengths down to an eighth of the
+    smearing.  The kernel is the difference of two terms of 2 e^{a^2} at most (a = kappa eta/2) over d, the slope over
+    d^2; in that unit FP32 leaves 4e-7 from the distance and its reciprocal powers, 5e-7 from erfcx (4 ulp), 3e-7 from the
+    exponentials and as much from the products: 2.5e-6 allowed."""
+    import torch
+    from scipy.special import erfcx
+
+    rng = np.random.default_rng(5)
+    n, N, h, eta = 600, (24, 20, 18), 0.5, 1.0
+    r = R.Rism(N, h, (0.0, 0.0, 0.0), method=getattr(R, "METHOD_" + method), precision=R.PREC_FP32, kappa=kappa,
+               lj_mode=R.LJ_NONE)
+    o = r.opts
+    r.set_solvent([0.75], [1.0], [0.1])
+    p0 = np.array([11, 9, 8])
+    u = rng.normal(size=(n, 3))
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    xyz = h * p0 + u * np.exp(rng.uniform(np.log(0.02), np.log(7.0), size=n))[:, None]
+    d = np.linalg.norm(xyz - h * p0, axis=1)
+    r.set_solute(xyz, np.ones(n), np.zeros(n), np.zeros(n))
+    G = torch.zeros((1, N[2], N[1], N[0]), dtype=torch.float64, device="cuda")
+    G[0, p0[2], p0[1], p0[0]] = 1.0
+    g = {k: v.cpu().numpy() for k, v in r.backward(None, None, G).items()}
+    r.close()
+    W = -o.k_e / (o.k_B * o.T) / (2.0 * o.eps_r) * 0.75
+    a, x, ex = 0.5 * kappa * eta, d / eta, np.exp(-((d / eta) ** 2))
+    E = 2.0 * np.exp(a * a) * np.exp(-kappa * d)
+    H0 = ex * (erfcx(x - a) + erfcx(x + a))
+    H1 = H0 - x * (2.0 * a * ex * (erfcx(x + a) - erfcx(x - a)) - 4.0 / np.sqrt(np.pi) * ex)
+    unit = 2.0 * np.exp(a * a) * abs(W)
+    dq = W * (E - H0) / d
+    dxyz = (-W * (E * (1.0 + kappa * d) - H1) / d ** 2 / d)[:, None] * (xyz - h * p0)
+    assert np.max(np.abs(g["q"] - dq) * d) / unit <= 2.5e-6
+    assert np.max(np.linalg.norm(g["xyz"] - dxyz, axis=1) * d ** 2) / unit <= 2.5e-6
