@@ -363,13 +363,15 @@ __device__ __forceinline__ bool point_box(const GridD& g, const SrcF& sf, float 
     return any;
 }
 
+constexpr int kFold = 64;
 // wpa warps per atom over the grid columns of its spheres: the erfc corrections (dq, G) within r_short, then the LJ
 // terms within the largest cut-off of the atom's sites.  A lane owns a column of a tile and goes down its chord, so x
 // and y offsets are fixed and the x, y forces take the column's sum once.  Per site the sums of G_u/d^12 and G_u/d^6
-// are kept (two sites per two-wide instruction); sigma and eps gradients follow from them at the end.  FP32 sums of one
-// column, folded into float pairs per tile.  UNI: one cut-off for all of an atom's sites.  FN: the short-range kernels by
-// their functions instead of the pieces.
-// Bound by issue and the latency of the cotangent loads (two CTAs per SM at 118 registers; three at 80 spill and are
+// are kept (two sites per two-wide instruction); sigma and eps gradients follow from them at the end.  FP32 sums of at
+// most kFold points of a column, folded into float pairs, so that rounding does not grow with the length of a column (all
+// of nz without a cut-off); a chord within a cut-off is mostly one fold.  UNI: one cut-off for all of an atom's sites.
+// FN: the short-range kernels by their functions instead of the pieces.
+// Bound by issue and the latency of the cotangent loads (two CTAs per SM at 121 registers; three at 80 spill and are
 // slower).  2,000 atoms on 128^3: 0.34 ms (1.02 ms with one CTA per atom that called erfc, erfcx and, in every thread,
 // the FP64 mixing derivatives); 55,000 atoms on 320x320x384, u and c: 7.7 ms (21.2).
 template <int NR, bool UNI, bool FN>
@@ -397,45 +399,48 @@ __global__ void __launch_bounds__(kNearT) k_adj_near(const __grid_constant__ Nea
             for (int t = sub; t < nt; t += a.wpa) {
                 const ColTile c = col_tile(g, sf, lo, hi, a.rs2, t, ntx, lane);
                 const float4* pw = a.w + c.at;
-                float dq = 0.f, rs = 0.f, rz = 0.f;
                 float fk = (float)c.k0;
+                for (int kb = c.k0; kb <= c.k1; kb += kFold) {
+                    const int ke = min(c.k1, kb + kFold - 1);
+                    float dq = 0.f, rs = 0.f, rz = 0.f;
 #pragma unroll 4
-                for (int kk = c.k0; kk <= c.k1; ++kk, pw += plane, fk += 1.f) {
-                    const float2 W = __ldg(reinterpret_cast<const float2*>(pw) + 1);  // Wc, Wh
-                    const float dz = (fk - sf.zh) - sf.zl;
-                    const float d2 = fmaf(dz, dz, c.dxy2);
-                    const bool ok = d2 < a.rs2 && d2 > 0.f;
-                    const float dd = ok ? d2 : 1.f;
-                    const float ri = rsqrt_approx(dd);
-                    const float wc = ok ? W.x : 0.f, wh = ok ? W.y : 0.f;
-                    float f0, f1;
-                    if (FN) {
-                        const float4 k = near_functions(dd * ri * a.xs, a.aa);
-                        // without a cotangent of h nothing of its kernel enters (it overflows at extreme screening)
-                        f0 = fmaf(wc, k.x, wh != 0.f ? wh * k.z : 0.f);
-                        f1 = fmaf(wc, k.y, wh != 0.f ? wh * k.w : 0.f);
-                    } else {
-                        const float u = dd * ri * a.tab_inv;
-                        // segment of u: adding 1.5 2^23 leaves round(u - 1/2) in the low bits of the sum
-                        const float sh = (u - 0.5f) + 12582912.0f;
-                        const int it = min(__float_as_int(sh) - 0x4B400000, kAdjTab - 1);
-                        const float tt = u - fminf(sh - 12582912.0f, (float)(kAdjTab - 1));
-                        auto piece = [&](int f) {
-                            const float4 k = tab[it][f];
-                            return fmaf(fmaf(fmaf(k.w, tt, k.z), tt, k.y), tt, k.x);
-                        };
-                        f0 = fmaf(wc, piece(0), wh * piece(2));
-                        f1 = fmaf(wc, piece(1), wh * piece(3));
+                    for (int kk = kb; kk <= ke; ++kk, pw += plane, fk += 1.f) {
+                        const float2 W = __ldg(reinterpret_cast<const float2*>(pw) + 1);  // Wc, Wh
+                        const float dz = (fk - sf.zh) - sf.zl;
+                        const float d2 = fmaf(dz, dz, c.dxy2);
+                        const bool ok = d2 < a.rs2 && d2 > 0.f;
+                        const float dd = ok ? d2 : 1.f;
+                        const float ri = rsqrt_approx(dd);
+                        const float wc = ok ? W.x : 0.f, wh = ok ? W.y : 0.f;
+                        float f0, f1;
+                        if (FN) {
+                            const float4 k = near_functions(dd * ri * a.xs, a.aa);
+                            // without a cotangent of h nothing of its kernel enters (it overflows at extreme screening)
+                            f0 = fmaf(wc, k.x, wh != 0.f ? wh * k.z : 0.f);
+                            f1 = fmaf(wc, k.y, wh != 0.f ? wh * k.w : 0.f);
+                        } else {
+                            const float u = dd * ri * a.tab_inv;
+                            // segment of u: adding 1.5 2^23 leaves round(u - 1/2) in the low bits of the sum
+                            const float sh = (u - 0.5f) + 12582912.0f;
+                            const int it = min(__float_as_int(sh) - 0x4B400000, kAdjTab - 1);
+                            const float tt = u - fminf(sh - 12582912.0f, (float)(kAdjTab - 1));
+                            auto piece = [&](int f) {
+                                const float4 k = tab[it][f];
+                                return fmaf(fmaf(fmaf(k.w, tt, k.z), tt, k.y), tt, k.x);
+                            };
+                            f0 = fmaf(wc, piece(0), wh * piece(2));
+                            f1 = fmaf(wc, piece(1), wh * piece(3));
+                        }
+                        dq = fmaf(-f0, ri, dq);
+                        const float rad = f1 * ri * ri * ri;
+                        rs += rad;
+                        rz = fmaf(dz, rad, rz);
                     }
-                    dq = fmaf(-f0, ri, dq);
-                    const float rad = f1 * ri * ri * ri;
-                    rs += rad;
-                    rz = fmaf(dz, rad, rz);
+                    ff_add(v[0].h, v[0].l, dq);
+                    ff_add(v[1].h, v[1].l, c.dxy2 < INFINITY ? c.dx * rs : 0.f);
+                    ff_add(v[2].h, v[2].l, c.dxy2 < INFINITY ? c.dy * rs : 0.f);
+                    ff_add(v[3].h, v[3].l, rz);
                 }
-                ff_add(v[0].h, v[0].l, dq);
-                ff_add(v[1].h, v[1].l, c.dxy2 < INFINITY ? c.dx * rs : 0.f);
-                ff_add(v[2].h, v[2].l, c.dxy2 < INFINITY ? c.dy * rs : 0.f);
-                ff_add(v[3].h, v[3].l, rz);
             }
         }
         if (live && a.gu4) {
@@ -467,72 +472,75 @@ __global__ void __launch_bounds__(kNearT) k_adj_near(const __grid_constant__ Nea
             for (int t = sub; t < nt; t += a.wpa) {
                 const ColTile c = col_tile(g, sf, lo, hi, rmax, t, ntx, lane);
                 const float4* pg = a.gu4 + c.at;
-                f32x2 s12[2 * NR], s6[2 * NR];
-#pragma unroll
-                for (int s = 0; s < 2 * NR; ++s) s12[s] = s6[s] = 0ull;
-                float fs = 0.f, fz = 0.f;
                 float fk = (float)c.k0;
+                for (int kb = c.k0; kb <= c.k1; kb += kFold) {
+                    const int ke = min(c.k1, kb + kFold - 1);
+                    f32x2 s12[2 * NR], s6[2 * NR];
+#pragma unroll
+                    for (int s = 0; s < 2 * NR; ++s) s12[s] = s6[s] = 0ull;
+                    float fs = 0.f, fz = 0.f;
 #pragma unroll 4
-                for (int kk = c.k0; kk <= c.k1; ++kk, pg += plane, fk += 1.f) {
-                    ulonglong2 gv[NR];  // loaded before the tests: the loads of the unrolled points run together
+                    for (int kk = kb; kk <= ke; ++kk, pg += plane, fk += 1.f) {
+                        ulonglong2 gv[NR];  // loaded before the tests: the loads of the unrolled points run together
 #pragma unroll
-                    for (int q = 0; q < NR; ++q) gv[q] = __ldg(reinterpret_cast<const ulonglong2*>(pg + q * M));
-                    const float dz = (fk - sf.zh) - sf.zl;
-                    const float d2 = fmaf(dz, dz, c.dxy2);
-                    // a point outside the cut-off, or on the atom, has no term whatever its cotangent is
-                    const bool ok = d2 < rmax && d2 > 0.f;
-                    float r2 = rcp_approx(ok ? d2 : 1.f);
-                    // the nearest points carry the sums, and their error counts seven times: there 1/d^2 takes what
-                    // the rounding of d^2 and of the reciprocal left
-                    if (__any_sync(0xffffffffu, ok && d2 < 4.f)) {
-                        const float e = dist2_rest(c.dx, c.dy, dz, (c.fx - sf.xh) - c.dx, (c.fy - sf.yh) - c.dy,
-                                                   (fk - sf.zh) - dz, sf, d2);
-                        r2 = fmaf(r2, fmaf(-d2, r2, 1.f) - e * r2, r2);
-                    }
-                    if (!ok) r2 = 0.f;
-                    f32x2 G[2 * NR];
+                        for (int q = 0; q < NR; ++q) gv[q] = __ldg(reinterpret_cast<const ulonglong2*>(pg + q * M));
+                        const float dz = (fk - sf.zh) - sf.zl;
+                        const float d2 = fmaf(dz, dz, c.dxy2);
+                        // a point outside the cut-off, or on the atom, has no term whatever its cotangent is
+                        const bool ok = d2 < rmax && d2 > 0.f;
+                        float r2 = rcp_approx(ok ? d2 : 1.f);
+                        // the nearest points carry the sums, and their error counts seven times: there 1/d^2 takes what
+                        // the rounding of d^2 and of the reciprocal left
+                        if (__any_sync(0xffffffffu, ok && d2 < 4.f)) {
+                            const float e = dist2_rest(c.dx, c.dy, dz, (c.fx - sf.xh) - c.dx, (c.fy - sf.yh) - c.dy,
+                                                       (fk - sf.zh) - dz, sf, d2);
+                            r2 = fmaf(r2, fmaf(-d2, r2, 1.f) - e * r2, r2);
+                        }
+                        if (!ok) r2 = 0.f;
+                        f32x2 G[2 * NR];
 #pragma unroll
-                    for (int q = 0; q < NR; ++q) {
-                        G[2 * q] = ok ? gv[q].x : 0ull;
-                        G[2 * q + 1] = ok ? gv[q].y : 0ull;
-                    }
-                    if (!UNI) {
+                        for (int q = 0; q < NR; ++q) {
+                            G[2 * q] = ok ? gv[q].x : 0ull;
+                            G[2 * q + 1] = ok ? gv[q].y : 0ull;
+                        }
+                        if (!UNI) {
+#pragma unroll
+                            for (int s = 0; s < 2 * NR; ++s) {
+                                const float2 q = up2(G[s]);
+                                G[s] = pk2(d2 < rc[2 * s] ? q.x : 0.f, d2 < rc[2 * s + 1] ? q.y : 0.f);
+                            }
+                        }
+                        const float r6 = r2 * r2 * r2, r12 = r6 * r6;
+                        const f32x2 R6 = pk2(r6, r6), R12 = pk2(r12, r12);
+                        f32x2 T12 = mul2(A[0], G[0]), T6 = mul2(B[0], G[0]);
+#pragma unroll
+                        for (int s = 1; s < 2 * NR; ++s) {
+                            T12 = fma2(A[s], G[s], T12);
+                            T6 = fma2(B[s], G[s], T6);
+                        }
 #pragma unroll
                         for (int s = 0; s < 2 * NR; ++s) {
-                            const float2 q = up2(G[s]);
-                            G[s] = pk2(d2 < rc[2 * s] ? q.x : 0.f, d2 < rc[2 * s + 1] ? q.y : 0.f);
+                            s12[s] = fma2(G[s], R12, s12[s]);
+                            s6[s] = fma2(G[s], R6, s6[s]);
                         }
-                    }
-                    const float r6 = r2 * r2 * r2, r12 = r6 * r6;
-                    const f32x2 R6 = pk2(r6, r6), R12 = pk2(r12, r12);
-                    f32x2 T12 = mul2(A[0], G[0]), T6 = mul2(B[0], G[0]);
-#pragma unroll
-                    for (int s = 1; s < 2 * NR; ++s) {
-                        T12 = fma2(A[s], G[s], T12);
-                        T6 = fma2(B[s], G[s], T6);
+                        const float2 p12 = up2(T12), p6 = up2(T6);
+                        // dLJ/dd / d, grid units
+                        const float lrad = fmaf(-12.f * (p12.x + p12.y), r6, 6.f * (p6.x + p6.y)) * (r6 * r2);
+                        fs += lrad;
+                        fz = fmaf(dz, lrad, fz);
                     }
 #pragma unroll
                     for (int s = 0; s < 2 * NR; ++s) {
-                        s12[s] = fma2(G[s], R12, s12[s]);
-                        s6[s] = fma2(G[s], R6, s6[s]);
+                        const float2 t12 = up2(s12[s]), t6 = up2(s6[s]);
+                        ff_add(x12[2 * s].h, x12[2 * s].l, t12.x);
+                        ff_add(x12[2 * s + 1].h, x12[2 * s + 1].l, t12.y);
+                        ff_add(x6[2 * s].h, x6[2 * s].l, t6.x);
+                        ff_add(x6[2 * s + 1].h, x6[2 * s + 1].l, t6.y);
                     }
-                    const float2 p12 = up2(T12), p6 = up2(T6);
-                    // dLJ/dd / d, grid units
-                    const float lrad = fmaf(-12.f * (p12.x + p12.y), r6, 6.f * (p6.x + p6.y)) * (r6 * r2);
-                    fs += lrad;
-                    fz = fmaf(dz, lrad, fz);
+                    ff_add(v[4].h, v[4].l, c.dxy2 < INFINITY ? c.dx * fs : 0.f);
+                    ff_add(v[5].h, v[5].l, c.dxy2 < INFINITY ? c.dy * fs : 0.f);
+                    ff_add(v[6].h, v[6].l, fz);
                 }
-#pragma unroll
-                for (int s = 0; s < 2 * NR; ++s) {
-                    const float2 t12 = up2(s12[s]), t6 = up2(s6[s]);
-                    ff_add(x12[2 * s].h, x12[2 * s].l, t12.x);
-                    ff_add(x12[2 * s + 1].h, x12[2 * s + 1].l, t12.y);
-                    ff_add(x6[2 * s].h, x6[2 * s].l, t6.x);
-                    ff_add(x6[2 * s + 1].h, x6[2 * s + 1].l, t6.y);
-                }
-                ff_add(v[4].h, v[4].l, c.dxy2 < INFINITY ? c.dx * fs : 0.f);
-                ff_add(v[5].h, v[5].l, c.dxy2 < INFINITY ? c.dy * fs : 0.f);
-                ff_add(v[6].h, v[6].l, fz);
             }
 #pragma unroll
             for (int q = 0; q < 4 * NR; ++q) {

@@ -401,3 +401,25 @@ def test_strong_screening_near_terms(R, kappa, method):
     dxyz = (-W * (E * (1.0 + kappa * d) - H1) / d ** 2 / d)[:, None] * (xyz - h * p0)
     assert np.max(np.abs(g["q"] - dq) * d) / unit <= 2.5e-6
     assert np.max(np.linalg.norm(g["xyz"] - dxyz, axis=1) * d ** 2) / unit <= 2.5e-6
+
+
+def test_long_columns_keep_small_terms(R):
+    """An LJ sum down a column of 8,000 points without a cut-off, one term of which is 2^26 times each of the others: added
+    up in FP32 alone the others (1.2e-4 of the sum) would be lost."""
+    import torch
+
+    nz, h, sig, eps = 8000, 0.5, 0.3, 0.1
+    d = 1.0 + h * np.arange(nz)
+    G = d ** 6
+    G[0] *= 2.0 ** 26
+    r = R.Rism((1, 1, nz), h, (0.0, 0.0, 0.0), method=R.METHOD_DIRECT, precision=R.PREC_FP32, kappa=0.0, lj_mode=R.LJ_NONE)
+    r.set_solvent([0.0], [sig], [eps])
+    r.set_solute([[0.0, 0.0, -1.0]], [0.0], [sig], [eps])
+    g = r.backward(torch.as_tensor(G.reshape(1, nz, 1, 1), device="cuda"), None, None)
+    g = {k: float(v.cpu().numpy()[0]) for k, v in g.items() if k in ("sigma", "eps")}
+    r.close()
+    A, B = 4.0 * eps * sig ** 12, 4.0 * eps * sig ** 6
+    ref = {"eps": float((G * (A / d ** 12 - B / d ** 6)).sum()) / (2.0 * eps),
+           "sigma": float((G * (12.0 * A / d ** 12 - 6.0 * B / d ** 6)).sum()) * 0.5 / sig}
+    for k, v in ref.items():
+        assert abs(g[k] - v) <= GRAD_TOL * abs(v), (k, g[k], v)
