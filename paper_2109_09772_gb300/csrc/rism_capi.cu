@@ -73,7 +73,7 @@ struct rism_ctx {
     double2* d_lra_atom = nullptr;
     int64_t lra_atom_cap = 0;
     double* d_lra_tot = nullptr;
-    size_t lra_tot_len = 0;
+    int64_t lra_tot_cap = 0;
     double* h_lra_tot = nullptr;  // pinned [3]
     float* d_lra_tab = nullptr;   // cubic pieces of the overlap integrals for lra_tab_key = (eta, kappa)
     double lra_tab_key[2] = {0.0, -1.0};
@@ -714,15 +714,14 @@ rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
     const int64_t need = (int64_t)lra_scratch_doubles(n, sms);
     if ((e = grow(c->lra_part_cap, need, buf(c->d_lra_part, need))) != cudaSuccess) return cuda_fail(c, e, "LRA scratch");
     if ((e = grow(c->lra_atom_cap, n, buf(c->d_lra_atom, n))) != cudaSuccess) return cuda_fail(c, e, "LRA atom sums");
-    if (lra_total_doubles(n) != c->lra_tot_len) {  // the counter's place depends on the length
-        const size_t len = lra_total_doubles(n);
-        c->lra_tot_len = 0;
-        int64_t cap = 0;
-        if ((e = alloc_once<PinnedMem>(c->h_lra_tot, 3)) != cudaSuccess ||
-            (e = grow(cap, (int64_t)len, buf(c->d_lra_tot, (int64_t)len))) != cudaSuccess ||
-            (e = cudaMemsetAsync(c->d_lra_tot, 0, sizeof(double) * len, c->st)) != cudaSuccess)
+    const int64_t len = (int64_t)lra_total_doubles(n);
+    if ((e = alloc_once<PinnedMem>(c->h_lra_tot, 3)) != cudaSuccess) return cuda_fail(c, e, "LRA totals");
+    if (len > c->lra_tot_cap) {
+        if ((e = grow(c->lra_tot_cap, len, buf(c->d_lra_tot, len))) != cudaSuccess ||
+            (e = cudaMemsetAsync(c->d_lra_tot, 0, sizeof(double) * len, c->st)) != cudaSuccess) {
+            c->lra_tot_cap = 0;
             return cuda_fail(c, e, "LRA totals");
-        c->lra_tot_len = len;
+        }
     }
     if (!c->d_lra_tab || c->lra_tab_key[0] != c->ph.eta || c->lra_tab_key[1] != c->ph.kappa) {
         if ((e = alloc_once(c->d_lra_tab, 8 * kLraTab)) != cudaSuccess) return cuda_fail(c, e, "LRA kernel table");

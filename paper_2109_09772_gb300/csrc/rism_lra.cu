@@ -287,8 +287,8 @@ __global__ void k_lra_gather(const SrcF* __restrict__ srcf, const int* __restric
 
 // Per atom: fixed-order sum of the chunk partials and the assembly of the two overlap sums (FP64).  Then the totals S_hh =
 // sum_a Q_a P_hh, S_hc = sum_a Q_a P_hc and Q: a tree per CTA, and the CTAs' sums in CTA order by the last one to finish
-// (a launch of one CTA for the totals took 17 us at 13,600 atoms).  tot: [3] totals, [3 + 3 CTAs] the CTAs' sums, then a
-// counter (zero between launches).
+// (a launch of one CTA for the totals took 17 us at 13,600 atoms).  tot: [3] totals, a counter (zero between launches), the
+// CTAs' sums.
 constexpr int kTotT = 256, kTotSub = 4, kTotAtoms = kTotT / kTotSub;  // threads per CTA and per atom
 __global__ void __launch_bounds__(kTotT) k_lra_atoms(const double* __restrict__ part, int n, int chunks, LraConst k,
                                                      const int* __restrict__ perm, const Geo* __restrict__ geo,
@@ -330,8 +330,8 @@ __global__ void __launch_bounds__(kTotT) k_lra_atoms(const double* __restrict__ 
         }
     };
     tree();
-    double* sums = tot + 3;
-    unsigned* done = reinterpret_cast<unsigned*>(sums + 3 * (size_t)gridDim.x);
+    unsigned* done = reinterpret_cast<unsigned*>(tot + 3);
+    double* sums = tot + 4;
     if (t == 0) {
         for (int m = 0; m < 3; ++m) sums[3 * (size_t)blockIdx.x + m] = red[m][0];
         __threadfence();
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kTotT) k_lra_atoms(const double* __restrict__ 
 
 }  // namespace
 
-size_t lra_total_doubles(int64_t n) { return 3 + 3 * (size_t)((n + kTotAtoms - 1) / kTotAtoms) + 1; }
+size_t lra_total_doubles(int64_t n) { return 4 + 3 * (size_t)((n + kTotAtoms - 1) / kTotAtoms); }
 
 size_t lra_scratch_doubles(int64_t n, int sms) {
     const int chunks = lra_chunks(n, sms);

@@ -9,7 +9,7 @@ namespace rism {
 // Source chunks of the pair kernel for n atoms on a device with `sms` SMs, and the FP64 scratch it needs.
 int lra_chunks(int64_t n, int sms);
 size_t lra_scratch_doubles(int64_t n, int sms);
-// Doubles of tot: the totals and their work space, zeroed once when allocated.
+// Doubles of tot: the totals and their work space, zeroed once when allocated (the same layout for every n).
 size_t lra_total_doubles(int64_t n);
 
 // Cubic pieces of the overlap integrals inside the short-range radius (host, kLraTab x 8 floats) for kappa > 0; they

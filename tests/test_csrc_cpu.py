@@ -94,3 +94,12 @@ def test_every_buffer_goes_through_the_grow_helper():
     for name, s in _code().items():
         n = len(re.findall(r"\bcudaMalloc(Host|Async|Managed)?\s*\(", s))
         assert n == (2 if name == "rism_internal.cuh" else 0), (name, n)
+
+
+def test_every_capacity_is_kept_beside_its_buffer():
+    """A buffer that serves one call after another only grows: its capacity is a member of the object that owns it, so a
+    smaller (or a repeated) need neither frees nor allocates."""
+    for name, s in _code().items():
+        for m in re.finditer(r"\bgrow(?:_with<\w+>)?\(\s*([^,;]+),[^;]*?\bbuf\(", s):
+            if name not in ("rism_grow.h", "rism_internal.cuh"):
+                assert re.match(r"(c|s)->\w+|A\.\w+", m.group(1)), f"{name}: {m.group(0)}"

@@ -131,3 +131,22 @@ def test_target_groups_tiles_and_totals(R, n):
         _check_atoms(a.cpu().numpy(), O.lra_atom_sums(p, np.arange(m)), f"{m} atoms")
         assert rel_l2(T, O.lra_integral(p)[0]) <= TOL
     r.close()
+
+
+def test_solutes_of_every_size_on_one_context(R):
+    """The work space of the totals serves smaller and larger solutes in any order: bit for bit what fresh contexts give."""
+    import torch
+
+    w = I.small_workload(n_atoms=700, n=(20, 20, 20), h=0.5, seed=52, ions=True, lj_rcut=4.0, net=1.0)
+    s = w.solute
+    r = R.from_workload(w, method=R.METHOD_TREECODE, precision=R.PREC_FP32)
+    for m in (300, 64, 700, 65, 1, 129, 700, 640):
+        part = I.Workload(w.name, I.Solute(s.xyz[:m], s.q[:m], s.sigma[:m], s.eps[:m]), w.solvent, w.grid, w.opts)
+        f = R.from_workload(part, method=R.METHOD_TREECODE, precision=R.PREC_FP32)
+        T, a = f.lra_integral(atom_sums=True)
+        r.set_solute(s.xyz[:m], s.q[:m], s.sigma[:m], s.eps[:m])
+        for _ in range(2):
+            T2, a2 = r.lra_integral(atom_sums=True)
+            assert np.array_equal(T, T2) and torch.equal(a, a2), m
+        f.close()
+    r.close()
