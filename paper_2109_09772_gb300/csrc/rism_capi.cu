@@ -16,6 +16,7 @@
 #include "rism_adjoint.h"
 #include "rism_validate.h"
 #include "rism_lra.h"
+#include "rism_order.h"
 #include "rism_kspace.h"
 
 using namespace rism;
@@ -629,62 +630,6 @@ rism_status rism_potential_batched(rism_ctx* const* ctxs, int32_t count, double*
     }
     return fail(c0, RISM_E_NOMEM, "list buffers kept growing");
 }
-
-namespace {
-
-uint32_t spread10(uint32_t v) {  // the 10 low bits of v to every third bit
-    v &= 0x3ffu;
-    v = (v | (v << 16)) & 0x030000ffu;
-    v = (v | (v << 8)) & 0x0300f00fu;
-    v = (v | (v << 4)) & 0x030c30c3u;
-    v = (v | (v << 2)) & 0x09249249u;
-    return v;
-}
-
-// Spatial order of the atoms for the all-space pair sum: cells of about 32 atoms over the atoms' bounding box,
-// the cells in Morton order, the atoms of a cell in index order (a stable counting sort, O(n)).  A warp then
-// takes nearby targets and a tile nearby sources, so the costly short-range branch of the pair term is taken by
-// whole warps or by none.  perm[k] = original index of the atom at position k.
-void lra_order(const double* raw, int64_t n, int* perm) {
-    double lo[3] = {raw[0], raw[1], raw[2]}, hi[3] = {raw[0], raw[1], raw[2]};
-    for (int64_t i = 1; i < n; ++i)
-        for (int d = 0; d < 3; ++d) {
-            lo[d] = std::min(lo[d], raw[6 * i + d]);
-            hi[d] = std::max(hi[d], raw[6 * i + d]);
-        }
-    double ext[3], vol = 1.0;
-    for (int d = 0; d < 3; ++d) {
-        ext[d] = std::max(hi[d] - lo[d], 1e-6);
-        vol *= ext[d];
-    }
-    const double side = std::cbrt(vol / (double)std::max<int64_t>(1, n / 32)), iside = 1.0 / side;
-    int nc[3];
-    for (int d = 0; d < 3; ++d) nc[d] = std::max(1, std::min(1024, (int)std::ceil(ext[d] / side)));
-    const int64_t ncell = (int64_t)nc[0] * nc[1] * nc[2];
-    std::vector<uint64_t> key((size_t)ncell);
-    for (int z = 0; z < nc[2]; ++z)
-        for (int y = 0; y < nc[1]; ++y)
-            for (int x = 0; x < nc[0]; ++x) {
-                const uint64_t m = spread10((uint32_t)x) | (spread10((uint32_t)y) << 1) | (spread10((uint32_t)z) << 2);
-                const int64_t lin = ((int64_t)z * nc[1] + y) * nc[0] + x;
-                key[(size_t)lin] = (m << 32) | (uint64_t)lin;
-            }
-    std::sort(key.begin(), key.end());
-    std::vector<int> rank((size_t)ncell), start((size_t)ncell + 1, 0);
-    for (int64_t r = 0; r < ncell; ++r) rank[(size_t)(key[(size_t)r] & 0xffffffffu)] = (int)r;
-    std::vector<int> cell((size_t)n);
-    for (int64_t i = 0; i < n; ++i) {
-        int cc[3];
-        for (int d = 0; d < 3; ++d)
-            cc[d] = std::min(nc[d] - 1, (int)((raw[6 * i + d] - lo[d]) * iside));  // never negative
-        cell[(size_t)i] = rank[(size_t)(((int64_t)cc[2] * nc[1] + cc[1]) * nc[0] + cc[0])];
-        ++start[(size_t)cell[(size_t)i] + 1];
-    }
-    for (int64_t r = 0; r < ncell; ++r) start[(size_t)r + 1] += start[(size_t)r];
-    for (int64_t i = 0; i < n; ++i) perm[start[(size_t)cell[(size_t)i]]++] = (int)i;
-}
-
-}  // namespace
 
 rism_status rism_lra_integral(rism_ctx* c, double* T, double* atom_sums) {
     if (!c) return RISM_E_INVALID;

@@ -103,3 +103,38 @@ def test_every_capacity_is_kept_beside_its_buffer():
         for m in re.finditer(r"\bgrow(?:_with<\w+>)?\(\s*([^,;]+),[^;]*?\bbuf\(", s):
             if name not in ("rism_grow.h", "rism_internal.cuh"):
                 assert re.match(r"(c|s)->\w+|A\.\w+", m.group(1)), f"{name}: {m.group(0)}"
+
+
+ORDER = r"""
+#include <stdio.h>
+#include <stdlib.h>
+#include "rism_order.h"
+int main() {
+    // extents along x, y, z and the number of atoms: a globule, a plane, lines short and long, one atom, two far apart
+    const double ext[][4] = {{40, 40, 40, 5000}, {300, 300, 0, 3000}, {1e4, 0, 0, 700}, {1e9, 0, 0, 64}, {1e13, 1e-3, 0, 700},
+                             {0, 1e200, 0, 33}, {1e308, 1e308, 0, 40}, {0, 0, 0, 1}, {0, 0, 0, 90}, {0, 0, 1e12, 2}};
+    for (const auto& e : ext) {
+        const int n = (int)e[3];
+        std::vector<double> raw(6 * (size_t)n, 0.0);
+        srand(7);
+        for (int i = 0; i < n; ++i)
+            for (int d = 0; d < 3; ++d)
+                raw[6 * (size_t)i + d] = e[d] * (i == 0 ? -0.5 : i == n - 1 ? 0.5 : rand() / (RAND_MAX + 1.0) - 0.5);
+        std::vector<int> perm((size_t)n, -1), seen((size_t)n, 0);
+        rism::lra_order(raw.data(), n, perm.data());
+        for (int p : perm) {
+            if (p < 0 || p >= n || seen[(size_t)p]++) return printf("extents %g %g %g\n", e[0], e[1], e[2]), 1;
+        }
+    }
+    return 0;
+}
+"""
+
+
+def test_spatial_order_of_any_solute(tmp_path):
+    """The order of the all-space pair sum is a permutation for solutes of any shape, also where a cell index computed in
+    floating point exceeds the integers (a line of atoms 1e13 A long)."""
+    src, exe = tmp_path / "order.cpp", tmp_path / "order"
+    src.write_text(ORDER)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wall", "-D_GLIBCXX_ASSERTIONS", "-I", CSRC, str(src), "-o", str(exe)])
+    subprocess.check_call([str(exe)])
