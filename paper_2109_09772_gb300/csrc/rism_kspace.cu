@@ -657,10 +657,11 @@ void kspace_charge_plan(const double* raw, int64_t n, KspaceSetup& s) {
         qmax = std::max(qmax, q);
         sum[(size_t)(i / kKA)] += q;
     }
-    // a power of two at least as large as every FP32 charge (1 for uncharged atoms; its reciprocal scales stay normal FP32 numbers)
+    // a power of two at least as large as every FP32 charge (1 for uncharged atoms), and no smaller than 2^-110, so that 256
+    // over it and it over 2^16 stay normal FP32 numbers
     int e = 0;
     std::frexp(qmax > 0.0 ? qmax : 0.5, &e);
-    s.qscale = std::ldexp(1.0, std::min(std::max(e, -110), 110));
+    s.qscale = std::ldexp(1.0, std::min(std::max(e, -110), 128));
     int64_t len = std::min<int64_t>(nch, kKBlock);
     for (; len > 1; len = len * 3 / 4) {
         double worst = 0.0;

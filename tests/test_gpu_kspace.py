@@ -163,3 +163,19 @@ def test_edge_cases(R):
     c, _, _ = r.asymptotics_k(0.0, c=True, h=False)
     assert float(c.abs().max()) == 0.0
     r.close()
+
+
+@pytest.mark.parametrize("power", [118, 60, -60])
+def test_charge_scale_is_exact(R, power):
+    """Solute charges times a power of two and site charges divided by it, up to the largest that FP32 holds: the same c(k)
+    bit for bit."""
+    import torch
+
+    w = I.small_workload(n_atoms=50, n=(18, 15, 14), h=0.9, seed=15, ions=False, lj_rcut=4.0, net=1.0)
+    s, v = w.solute, w.solvent
+    r = R.from_workload(w, method=R.METHOD_DIRECT, precision=R.PREC_FP32)
+    want = r.asymptotics_k(0.0, c=True, h=False)[0]
+    r.set_solvent(v.q * 2.0 ** -power, v.sigma, v.eps)
+    r.set_solute(s.xyz, s.q * 2.0 ** power, s.sigma, s.eps)
+    assert torch.equal(r.asymptotics_k(0.0, c=True, h=False)[0], want)
+    r.close()
