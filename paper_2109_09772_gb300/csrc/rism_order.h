@@ -34,13 +34,16 @@ inline void lra_order(const double* raw, int64_t n, int* perm) {
         ext[d] = std::max(hi[d] - lo[d], 1e-6);
         vol *= ext[d];
     }
-    const double side = std::cbrt(vol / (double)std::max<int64_t>(1, n / 32)), iside = 1.0 / side;
+    if (!std::isfinite(vol)) {  // atoms 1e100 A apart: no two of them are near, any order serves
+        for (int64_t i = 0; i < n; ++i) perm[i] = (int)i;
+        return;
+    }
+    const double side = std::cbrt(vol / (double)std::max<int64_t>(1, n / 32));
     int nc[3];
+    double inv[3];  // cells per A: 1 / side, or what 1,024 cells allow over the length of a thin solute
     for (int d = 0; d < 3; ++d) {
-        // compared before the conversion to an integer: a thin solute's cells are so small that their number along its
-        // length can exceed every integer type
-        const double k = std::ceil(ext[d] / side);
-        nc[d] = k >= 1024.0 ? 1024 : (k >= 1.0 ? (int)k : 1);
+        nc[d] = (int)std::max(1.0, std::min(1024.0, std::ceil(ext[d] / side)));
+        inv[d] = std::min(1.0 / side, nc[d] / ext[d]);
     }
     const int64_t ncell = (int64_t)nc[0] * nc[1] * nc[2];
     std::vector<uint64_t> key((size_t)ncell);
@@ -57,10 +60,8 @@ inline void lra_order(const double* raw, int64_t n, int* perm) {
     std::vector<int> cell((size_t)n);
     for (int64_t i = 0; i < n; ++i) {
         int cc[3];
-        for (int d = 0; d < 3; ++d) {
-            const double k = (raw[6 * i + d] - lo[d]) * iside;  // never negative
-            cc[d] = k < nc[d] - 1 ? (int)k : nc[d] - 1;
-        }
+        for (int d = 0; d < 3; ++d)
+            cc[d] = std::min(nc[d] - 1, (int)((raw[6 * i + d] - lo[d]) * inv[d]));  // between 0 and nc[d]
         cell[(size_t)i] = rank[(size_t)(((int64_t)cc[2] * nc[1] + cc[1]) * nc[0] + cc[0])];
         ++start[(size_t)cell[(size_t)i] + 1];
     }
