@@ -712,7 +712,7 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     const int nseg = seg_per_row * g.ny * g.nz;
     const int ablocks = (n + kAT * kAPT - 1) / (kAT * kAPT);
     // enough CTAs to fill the GPU several times; at most one per row segment
-    int chunks = (4 * 152 + ablocks - 1) / ablocks;
+    int chunks = (4 * sm_count() + ablocks - 1) / ablocks;
     chunks = max(1, min(chunks, min(nseg, 256)));
     const int tchunks = tree && o.method == RISM_METHOD_TREECODE ? tree_adjoint_chunks(n) : 0;
     const int64_t need_part = (int64_t)max(chunks, tchunks) * n * 4;
@@ -733,9 +733,9 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
         }
     wc.e2h = (float)(2.0 * ph.ea2);
     wc.e2l = (float)(2.0 * ph.ea2 - (double)wc.e2h);
-    if (ph.S <= 2) k_adj_weights<2><<<8 * 152, 256, 0, st>>>(M, ph.S, g_u, g_c, g_h, wc, s->w, s->gu4);
-    else if (ph.S <= 4) k_adj_weights<4><<<8 * 152, 256, 0, st>>>(M, ph.S, g_u, g_c, g_h, wc, s->w, s->gu4);
-    else k_adj_weights<8><<<8 * 152, 256, 0, st>>>(M, ph.S, g_u, g_c, g_h, wc, s->w, s->gu4);
+    if (ph.S <= 2) k_adj_weights<2><<<8 * sm_count(), 256, 0, st>>>(M, ph.S, g_u, g_c, g_h, wc, s->w, s->gu4);
+    else if (ph.S <= 4) k_adj_weights<4><<<8 * sm_count(), 256, 0, st>>>(M, ph.S, g_u, g_c, g_h, wc, s->w, s->gu4);
+    else k_adj_weights<8><<<8 * sm_count(), 256, 0, st>>>(M, ph.S, g_u, g_c, g_h, wc, s->w, s->gu4);
     FarAdjArgs fa;
     fa.nx = g.nx;
     fa.ny = g.ny;
@@ -791,8 +791,8 @@ rism_status adjoint_run(AdjointState* s, TreeState* tree, const DevTables& t, co
     na.out = s->near;
     // enough warps for 64 per SM: few atoms get several warps each
     na.wpa = 1;
-    while (na.wpa < kNearT / 32 && (int64_t)n * na.wpa < 64 * 152) na.wpa *= 2;
-    const int nctas = (int)std::min<int64_t>(((int64_t)n * na.wpa + kNearT / 32 - 1) / (kNearT / 32), 4 * 152);
+    while (na.wpa < kNearT / 32 && (int64_t)n * na.wpa < 64 * (int64_t)sm_count()) na.wpa *= 2;
+    const int nctas = (int)std::min<int64_t>(((int64_t)n * na.wpa + kNearT / 32 - 1) / (kNearT / 32), 4 * sm_count());
     const bool uni = o.lj_mode != RISM_LJ_TOL;
     if (pieces) near_launch<false>(na, ph.S, uni, nctas, st);
     else near_launch<true>(na, ph.S, uni, nctas, st);

@@ -761,12 +761,12 @@ cudaError_t run_direct(const GridD& g, const Phys& ph, const DevTables& t, int p
     if (prec == RISM_PREC_FP64) {
         // one point per lane where four would be fewer than three waves of CTAs (200 atoms, two sites, one against four
         // points: 32^3, 64 CTAs, 0.45 / 0.90 ms; 56^3, 392 CTAs, 1.79 / 1.94; 64^3, 512 CTAs, 2.46 / 2.41; 80^3 4.39 / 4.08)
-        if (ctas >= 3 * 152) return run_direct64<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
+        if (ctas >= 3 * (int64_t)sm_count()) return run_direct64<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
         return run_direct64<SM, 1, DU, DH>(g, ph, t, o, wl, dbg, st);
     }
     // four points per lane share an atom's y and z terms, but only where that still leaves a few waves of CTAs (2,000
     // atoms, 128^3, 4,096 CTAs: 2.30 against 2.61 ms; 500 atoms, 64^3, 512 CTAs: 0.47 against 0.39)
-    if (ctas >= 1824) return run_direct32<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
+    if (ctas >= 12 * (int64_t)sm_count()) return run_direct32<SM, 4, DU, DH>(g, ph, t, o, wl, dbg, st);
     return run_direct32<SM, 2, DU, DH>(g, ph, t, o, wl, dbg, st);
 }
 

@@ -86,6 +86,16 @@ cudaError_t raise_dyn_smem(F* kernel, size_t bytes) {
     return e;
 }
 
+// SMs of the device (one kind of device per process).
+inline int sm_count() {
+    static const int n = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
+    }();
+    return n;
+}
+
 // Device and page-locked host memory.  A failed allocation is reported by its return value alone: the runtime's record of
 // it is cleared, or the error check of the next launch would report it again.
 struct DeviceMem {

@@ -3040,8 +3040,6 @@ struct VShape {
     static constexpr int FT = FarShape<NX, NY, NZ, PF>::NTP, NTN = NearShape<NX, NY, NZ>::NTP;
 };
 
-int sm_count();
-
 template <int V, int SM, bool DU, bool DH>
 struct Kern {
     using S = VShape<V>;
@@ -3201,17 +3199,6 @@ constexpr int kMaxCells = (1 << 21) + 1;  // 8^7 + 1
 rism_status cuda_err(std::string& err, cudaError_t e, const char* what) {
     err = std::string(what) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? RISM_E_NOMEM : RISM_E_CUDA;
-}
-
-int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 1;
-    }
-    return n;
 }
 
 // Host allocations for one solute (never inside a stream capture).

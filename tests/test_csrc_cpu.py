@@ -138,3 +138,9 @@ def test_spatial_order_of_any_solute(tmp_path):
     src.write_text(ORDER)
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wall", "-D_GLIBCXX_ASSERTIONS", "-I", CSRC, str(src), "-o", str(exe)])
     subprocess.check_call([str(exe)])
+
+
+def test_no_sm_count_in_the_code():
+    """Grids and dispatch rules take the number of SMs from the device."""
+    for name, s in _code().items():
+        assert not re.search(r"\b(152|1824)\b", s), name
