@@ -15,9 +15,10 @@
 // exact form of the far-field simplification eq. (tcfexp) of Sec. 2.4.2.
 //
 // Data movement: atoms are streamed through shared memory in tiles of T by
-// bulk TMA copies (cp.async.bulk + mbarrier, double-buffered, bounded waits);
-// every thread owns a strip of P consecutive x points at one (y, z) and reads
-// each atom as a shared-memory broadcast.
+// bulk TMA copies (cp.async.bulk + mbarrier, double-buffered, bounded waits).
+// A warp owns a compact block of 2P x 4 x 4 points, a thread P consecutive x
+// points of it, and reads each atom (FP32: each pair of atoms) as a
+// shared-memory broadcast.
 #include <cmath>
 #include <vector>
 
@@ -188,7 +189,8 @@ void short_range_table(const Phys& ph, double h, float4* tab) {
 // Taylor pieces: in t = (u - middle) with u = d kTab64 / r_short, |t| <= 1/2.  With E = e^{-x^2} and H_k the Hermite
 // polynomials, E^(k) = (-1)^k H_k E; F_c' = -(2/sqrt(pi)) E; and F_h = G- + G+ with G-+ = e^{a^2 -+ 2ax} erfc(x -+ a),
 // G-+' = -+ 2a G-+ - (2/sqrt(pi)) E, differentiated term by term.  Eight terms leave less than 1e-16 (the segments are
-// 0.0234 eta wide at r_short = 6 eta).
+// 0.0234 eta wide at r_short = 6 eta): absolute, where the library's functions are good to an ulp of their value.  What
+// they are subtracted from (q/d and its screened form) has that absolute error already.
 void short_range_table64(const Phys& ph, double* tab) {
     const double a = ph.a, dx = ph.rs / ph.eta / kTab64, tsp = 2.0 / std::sqrt(3.14159265358979323846);
     for (int s = 0; s < kTab64; ++s) {

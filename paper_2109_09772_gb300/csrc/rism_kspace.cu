@@ -411,11 +411,12 @@ __device__ __forceinline__ void zero_fill(const KSumArgs& a, const KItem& it, in
 }
 
 // What bounds it (13,600 atoms, 224x192x160, the whole half spectrum: 256 rows x 31,428 columns x 13,600 atoms x six
-// products, 1.3e12 FP16 multiplications): 0.80 ms, of which the products are 0.59 ms at the tensor cores' rate (12
-// MMAs of 112 clocks per chunk against 1,860 measured; the builders need about as long), the running sums 0.14 ms and
-// the outputs (444 MB) 0.07 ms.  The form it replaces, complex FP32 multiply-adds on the FMA pipe over twice the
-// columns, took 10.1 ms.  Columns 4 x 64: narrower items read the row operand more often per product.  The two
-// accumulators take all 512 TMEM columns, so the read-back of an item does not overlap the products of the next.
+// products, 1.3e12 FP16 operations): 0.95 ms.  The items are 56 pairs wide there (224 columns), two to a CTA, 425
+// chunks each: at 1,860 clocks a chunk 0.76 ms, of which the tensor cores need 1,344 (12 MMAs of 128 x 224 x 16, 112
+// clocks each: 0.55 ms) and the builders about as long.  The rest, 0.19 ms, is the read-back: the running sums of an
+// item's blocks and the outputs (444 MB).  The form it replaces, complex FP32 multiply-adds on the FMA pipe over twice
+// the columns, took 10.1 ms.  Narrower items read the row operand more often per product.  The two accumulators take
+// all 512 TMEM columns, so the read-back of an item does not overlap the products of the next.
 __global__ void __launch_bounds__(kKThreads, 1) k_ksum(const __grid_constant__ KSumArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* sA = smem;                              // [stage][slice][atom/8][row][8 halves]
@@ -657,8 +658,8 @@ void kspace_charge_plan(const double* raw, int64_t n, KspaceSetup& s) {
         qmax = std::max(qmax, q);
         sum[(size_t)(i / kKA)] += q;
     }
-    // a power of two at least as large as every FP32 charge (1 for uncharged atoms), and no smaller than 2^-110, so that 256
-    // over it and it over 2^16 stay normal FP32 numbers
+    // a power of two at least as large as every FP32 charge (1 for uncharged atoms), and no smaller than 2^-110, so that
+    // 256 over it and it over 2^16 stay normal FP32 numbers
     int e = 0;
     std::frexp(qmax > 0.0 ? qmax : 0.5, &e);
     s.qscale = std::ldexp(1.0, std::min(std::max(e, -110), 128));

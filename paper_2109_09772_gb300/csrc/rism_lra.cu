@@ -15,8 +15,8 @@
 // sums, sum q/R, sum q e^{-kappa R}/R and sum q e^{-kappa R} (one rsqrt and one ex2 per pair), and short-range
 // remainders that fall below 1e-15 relative beyond R = 6 sqrt(2) eta.  Within that radius both integrals are
 // smooth functions of R and the pair takes them whole from cubic pieces built in FP64 (the closed forms' terms cancel
-// there by several bits).  At R = 0 (an atom with itself) the limits I_hc(0) = 8 pi erfcx(b)/kappa and I_hh(0) = (8 pi/kappa) erfcx(b) + 16 pi sigma b erfcx(b)
-// - 16 sigma sqrt(pi) apply.
+// there by several bits).  At R = 0 (an atom with itself) the limits I_hc(0) = 8 pi erfcx(b)/kappa and I_hh(0) = (8
+// pi/kappa) erfcx(b) + 16 pi sigma b erfcx(b) - 16 sigma sqrt(pi) apply.
 //
 //   k_lra_gather: the source table in the spatial order chosen on the host (cells of about 32 atoms in Morton
 //                 order), so that a warp's targets and a tile's sources are each close together and the
